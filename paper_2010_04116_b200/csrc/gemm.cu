@@ -24,13 +24,13 @@
 
 #include "common.cuh"
 #include "gemm.h"
+#include "gemm_dev.cuh"
 
 namespace il {
 
 constexpr int BM = 128;                          // rows of A (and of the accumulator) held by one CTA
 constexpr int TILE_M = 2 * BM;                   // rows of the output tile of a CTA pair
 constexpr int BN = 256;                          // columns of the output tile; each CTA stages half of B
-constexpr int BK = 64;
 constexpr int A_BYTES = BM * BK * 2;             // 16 KB
 constexpr int B_BYTES = (BN / 2) * BK * 2;       // 16 KB
 constexpr int TMEM_COLS = 2 * BN;                // 512 columns: two accumulators
@@ -51,47 +51,6 @@ constexpr int STG_LD = 32;                       // floats per row of an epilogu
 constexpr int STG_BYTES = EPI_WARPS * 32 * STG_LD * 4;
 template <int NT> constexpr int smem_bytes() {
   return TileCfg<NT>::STAGES * TileCfg<NT>::STAGE_BYTES + 1024 /*alignment slack*/ + BAR_BYTES + STG_BYTES;
-}
-
-struct GemmDev {
-  int M, N, K;
-  int tiles_m, tiles_n;
-  int group_m;                   // row blocks per group of the tile order
-  int split_k, kb_per_split;     // work unit = (tile, k-range); split_k > 1 adds into C with red.add
-  void* C;
-  int ldc;
-  void* C2;
-  const float* bias;
-  const float* resid;
-  const bf16* aux;
-  int ld_aux, aux_rows;
-  float* colsum;                 // EPI_BF16_DGELU: += column sums of the output over rows < aux_rows (or NULL)
-  int accumulate;
-  const int* targets;
-  float* part_max;
-  float* part_sum;
-  int part_ld;
-  float* tgt_logit;
-  const float* lse;
-  float scale;
-  int col0;
-  const float* rowscale;
-  int store_exp;
-  unsigned* err;
-};
-
-// Tile order: groups of group_m row blocks are swept across all column blocks before the next group starts, so
-// that the pairs running at the same time share a small set of A rows and the whole of B in L2.  B is read from
-// DRAM once per group, A once in total: the host makes the group as tall as the matrix when all of A fits in
-// L2 beside the streams passing through it (the heads' [Ntok, V, d] projection: W would otherwise be read four
-// times), and 8 row blocks otherwise.
-__device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int group_m, int& m_blk, int& n_blk) {
-  const int per_group = group_m * tiles_n;
-  const int g = t / per_group;
-  const int within = t - g * per_group;
-  const int gm = min(group_m, tiles_m - g * group_m);
-  m_blk = g * group_m + within % gm;
-  n_blk = within / gm;
 }
 
 struct RowState {   // per-thread state carried across the 32-column chunks of one tile row (EPI_LSE)
@@ -156,116 +115,6 @@ __device__ __forceinline__ void epilogue_rowwise(const GemmDev& p, int col, floa
     const int tj = st.tgt - (p.col0 + col);
 #pragma unroll
     for (int j = 0; j < 32; ++j) v[j] = (ex2_fast((v[j] - l) * 1.4426950408889634f) - (j == tj ? 1.0f : 0.0f)) * p.scale;
-  }
-}
-
-// Element-wise part of the epilogue, after the 32 x 32 chunk has been transposed through shared memory: a
-// lane now holds 4 consecutive columns (gcol..gcol+3) of row grow, 8 lanes cover 128 contiguous bytes of
-// fp32 output (64 of bf16), so every global access is coalesced.  The loads of the second operand
-// (residual, saved pre-activation, or C itself when accumulating) are split from the stores so that all of
-// a chunk's loads are in flight before the first store (C may alias the residual).
-template <int EPI>
-__device__ __forceinline__ float4 epilogue_load4(const GemmDev& p, int grow, int arow, int gcol) {
-  float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
-  const bool vec = (gcol + 4 <= p.N);
-  if constexpr (EPI == EPI_F32_RESID || EPI == EPI_F32) {
-    const float* add = nullptr;
-    if constexpr (EPI == EPI_F32_RESID) add = p.resid + (size_t)grow * p.ldc + gcol;
-    else if (p.accumulate) add = reinterpret_cast<const float*>(p.C) + (size_t)grow * p.ldc + gcol;
-    if (add) {
-      if (vec) {
-        e = *reinterpret_cast<const float4*>(add);
-      } else {
-        e.x = add[0];
-        if (gcol + 1 < p.N) e.y = add[1];
-        if (gcol + 2 < p.N) e.z = add[2];
-      }
-    }
-  } else if constexpr (EPI == EPI_BF16_DGELU) {
-    const bf16* h = p.aux + (size_t)arow * p.ld_aux + gcol;   // arow = grow % aux_rows
-    if (vec) {
-      const uint2 hv = *reinterpret_cast<const uint2*>(h);
-      const float2 h0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hv.x));
-      const float2 h1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hv.y));
-      e = make_float4(h0.x, h0.y, h1.x, h1.y);
-    } else {
-      e.x = __bfloat162float(h[0]);
-      if (gcol + 1 < p.N) e.y = __bfloat162float(h[1]);
-      if (gcol + 2 < p.N) e.z = __bfloat162float(h[2]);
-    }
-  }
-  return e;
-}
-
-template <int EPI>
-__device__ __forceinline__ void epilogue_store4(const GemmDev& p, int grow, int gcol, float4 a, float4 e) {
-  const bool vec = (gcol + 4 <= p.N);
-  float v[4] = {a.x, a.y, a.z, a.w};
-  if constexpr (EPI == EPI_BF16 || EPI == EPI_BF16_GELU || EPI == EPI_F32_RESID) {
-    if (p.bias) {
-      if (vec) {
-        const float4 b = __ldg(reinterpret_cast<const float4*>(p.bias + gcol));
-        v[0] += b.x; v[1] += b.y; v[2] += b.z; v[3] += b.w;
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (gcol + j < p.N) v[j] += __ldg(p.bias + gcol + j);
-      }
-    }
-  }
-  if constexpr (EPI == EPI_BF16 || EPI == EPI_BF16_GELU || EPI == EPI_DZ || EPI == EPI_BF16_DGELU || EPI == EPI_LSE) {
-    bf16* c = reinterpret_cast<bf16*>(p.C) + (size_t)grow * p.ldc + gcol;
-    if constexpr (EPI == EPI_BF16_DGELU) {
-      v[0] *= e.x; v[1] *= e.y; v[2] *= e.z; v[3] *= e.w;
-      if (p.colsum && grow < p.aux_rows) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (gcol + j < p.N) atomicAdd(p.colsum + gcol + j, v[j]);
-      }
-    }
-    float y[4] = {0.f, 0.f, 0.f, 0.f};
-    if constexpr (EPI == EPI_BF16_GELU) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float d;
-        gelu_tanh_both(v[j], y[j], d);
-        v[j] = d;                                   // C receives gelu'(pre), C2 gelu(pre)
-      }
-    }
-    if (vec) {
-      uint2 o;
-      o.x = pack_bf16x2(v[0], v[1]);
-      o.y = pack_bf16x2(v[2], v[3]);
-      *reinterpret_cast<uint2*>(c) = o;
-      if constexpr (EPI == EPI_BF16_GELU) {
-        uint2 g;
-        g.x = pack_bf16x2(y[0], y[1]);
-        g.y = pack_bf16x2(y[2], y[3]);
-        *reinterpret_cast<uint2*>(reinterpret_cast<bf16*>(p.C2) + (size_t)grow * p.ldc + gcol) = g;
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (gcol + j < p.N) {
-          c[j] = __float2bfloat16(v[j]);
-          if constexpr (EPI == EPI_BF16_GELU)
-            (reinterpret_cast<bf16*>(p.C2) + (size_t)grow * p.ldc + gcol)[j] = __float2bfloat16(y[j]);
-        }
-    }
-  } else if constexpr (EPI == EPI_F32_RESID || EPI == EPI_F32) {
-    float* c = reinterpret_cast<float*>(p.C) + (size_t)grow * p.ldc + gcol;
-    v[0] += e.x; v[1] += e.y; v[2] += e.z; v[3] += e.w;
-    if (EPI == EPI_F32 && p.split_k > 1) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (gcol + j < p.N) atomicAdd(c + j, v[j]);
-    } else if (vec) {
-      *reinterpret_cast<float4*>(c) = make_float4(v[0], v[1], v[2], v[3]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (gcol + j < p.N) c[j] = v[j];
-    }
   }
 }
 
@@ -755,6 +604,8 @@ cudaError_t gemm_init() {
                                    nt == 2 ? smem_bytes<2>() : smem_bytes<1>());
           if (e != cudaSuccess) return e;
         }
+  e = gemm_small_init();
+  if (e != cudaSuccess) return e;
   g_attr_done[dev] = true;
   return cudaSuccess;
 }
@@ -780,8 +631,7 @@ bool tma_encode_f32(CUtensorMap* tm, const void* ptr, int rank, const unsigned l
   return tma_encode_any(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ptr, rank, dims, strides_bytes, box);
 }
 
-// rows = extent of the operand's own index (M or N), kdim = contraction extent, box_rows = tile rows.
-static bool encode_operand(CUtensorMap* tm, const GemmOperand& op, int rows, int kdim, int box_rows) {
+bool encode_gemm_operand(CUtensorMap* tm, const GemmOperand& op, int rows, int kdim, int box_rows) {
   cuuint64_t dims[2], strides[1];
   cuuint32_t box[2], estr[2] = {1, 1};
   if (!op.mn_major) {            // memory [rows, kdim], k contiguous
@@ -798,16 +648,80 @@ static bool encode_operand(CUtensorMap* tm, const GemmOperand& op, int rows, int
   return r == CUDA_SUCCESS;
 }
 
+// Which kernel and tile, from a model of each one's time in microseconds.  The constants are measured (back-to-back
+// launches of the shapes of a training step from 256 to 16384 tokens, d 128 to 2560); the model is within about 15 % of
+// the measurements and the choice within 10 % of the best of all candidates on nearly all of them.
+//   paired, 256 x 256: 0.283 us per slab alone, 0.345 with all pairs busy; a wave costs its main loop or its epilogue,
+//     whichever is longer (the accumulators alternate).
+//   paired, 256 x 512: 0.55 / 0.64 per slab (of twice the columns), the epilogue is exposed.  Taken up to 10 % behind
+//     the square tile: it moves a quarter fewer operand bytes, which counts beside other streams and under the power cap.
+//   128 x 128 / 128 x 64: 0.26 / 0.245 per slab while each CTA has an SM to itself, 0.46 / 0.33 with two per SM.
+// max_atomic_split > 1 (EPI_F32 into a zeroed output): the paired kernel may split the contraction over up to that
+// many units that add with red.global.add; 3 us for the zeroing pass.
+GemmPlan gemm_plan(int M, int N, int K, int a_mn, int b_mn, int epi, int num_sms, int max_atomic_split) {
+  const int slabs = (K + BK - 1) / BK, pairs = num_sms / 2;
+  // epilogue of a 256 x 256 tile in steady state / exposed after the last tile, by epilogue
+  static const float EPI_STEADY[EPI_COUNT] = {5.0f, 8.2f, 10.0f, 9.5f, 5.5f, 7.0f, 6.0f};
+  static const float EPI_LAST[EPI_COUNT] = {0.8f, 3.2f, 3.2f, 4.2f, 3.0f, 2.0f, 2.0f};
+  GemmPlan best{0, 1, 1, 1, 1e30f};
+  for (int nt = 1; nt <= 2; ++nt) {
+    if (nt == 2 && N <= BN) break;
+    const int tiles = ((M + TILE_M - 1) / TILE_M) * ((N + nt * BN - 1) / (nt * BN));
+    for (int s = 1; s <= (max_atomic_split > 1 ? max_atomic_split : 1); ++s) {
+      if (s > 1 && slabs / s < 16) break;
+      const int per = (slabs + s - 1) / s, units = tiles * s, waves = (units + pairs - 1) / pairs;
+      const float load = units < pairs ? (float)units / pairs : 1.0f;
+      const float main = per * (nt == 1 ? 0.283f + 0.062f * load : 0.55f + 0.09f * load);
+      float t;
+      if (nt == 1) t = 4.5f + (waves - 1) * (main > EPI_STEADY[epi] ? main : EPI_STEADY[epi]) + main + EPI_LAST[epi];
+      else t = 0.9f * (4.5f + waves * (main + 1.1f * EPI_STEADY[epi]) + EPI_LAST[epi]);
+      if (s > 1) t += 3.0f;
+      if (t < best.us * 0.98f) best = GemmPlan{0, 1, nt, s, t};
+    }
+  }
+  if (!gemm_small_supported(a_mn, b_mn, epi)) return best;
+  // epilogue of a 128 x 128 / 128 x 64 tile
+  static const float EPI_SMALL[2][EPI_COUNT] = {{0.6f, 2.2f, 5.0f, 5.0f, 3.0f, 0.f, 0.f}, {0.3f, 1.0f, 1.6f, 2.2f, 1.0f, 0.f, 0.f}};
+  for (int tn = 64; tn <= 128; tn += 64) {
+    const long long tiles = (long long)((M + 127) / 128) * ((N + tn - 1) / tn);
+    if (tiles > 16ll * num_sms) continue;
+    for (int s = 1; s <= 8; s *= 2) {
+      if (s > 1 && slabs < 2 * s) break;
+      const int per = (slabs + s - 1) / s;
+      const long long ctas = tiles * s;
+      const float e = EPI_SMALL[tn == 64][epi] / s;
+      const int room = s == 8 ? num_sms * 2 / 3 : s == 4 ? num_sms * 5 / 6 : num_sms;   // wide clusters do not pack every SM
+      float t = 3.2f + (s == 1 ? 0.f : s == 8 ? 3.0f : 2.0f);
+      if (ctas <= room) {
+        t += per * (tn == 64 ? 0.245f : 0.26f) + e;
+      } else {
+        const int rounds = (int)((ctas + 2 * room - 1) / (2 * room));
+        t += rounds * (per * (tn == 64 ? 0.33f : 0.46f) + e) + 1.0f + 3.0f * (rounds - 1);
+      }
+      if (t < best.us * 0.98f) best = GemmPlan{tn, s, 1, 1, t};
+    }
+  }
+  return best;
+}
+
 cudaError_t gemm_launch(const GemmArgs& a, unsigned* err_word, int num_sms, cudaStream_t stream) {
   cudaError_t e = gemm_init();
   if (e != cudaSuccess) return e;
   if (a.M <= 0 || a.N <= 0 || a.K <= 0 || !a.A.ptr || !a.B.ptr || !err_word) return cudaErrorInvalidValue;
   if ((a.A.ld % 8) || (a.B.ld % 8) || ((uintptr_t)a.A.ptr % 16) || ((uintptr_t)a.B.ptr % 16)) return cudaErrorInvalidValue;
-  // Tile width.  256 x 512 tiles cut the operand bytes per product by a quarter but expose most of the epilogue,
-  // so they pay when the main loop of a tile is long (K) and the output is at least one such tile wide.
-  int nt = a.tile_blocks;
-  if (nt < 1 || nt > 2) nt = (a.N > BN && a.K >= 2048) ? 2 : 1;
-  if (a.N <= BN) nt = 1;
+  GemmPlan plan = gemm_plan(a.M, a.N, a.K, a.A.mn_major, a.B.mn_major, a.epilogue, num_sms, 0);
+  const bool atomic_split = a.split_k > 1 && a.epilogue == EPI_F32 && !a.accumulate;
+  if (a.tile_blocks > 0 || atomic_split) {       // the paired kernel, as asked for
+    plan.tn = 0;
+    plan.nt = a.tile_blocks == 1 || a.tile_blocks == 2 ? a.tile_blocks : (a.N > BN && a.K >= 2048) ? 2 : 1;
+    if (a.N <= BN) plan.nt = 1;
+  } else if (a.tile_blocks < 0) {
+    plan.tn = -a.tile_blocks & 64 ? 64 : 128;
+    plan.split = -a.tile_blocks & 15;
+    if (plan.split != 1 && plan.split != 2 && plan.split != 4 && plan.split != 8) return cudaErrorInvalidValue;
+    if (!gemm_small_supported(a.A.mn_major, a.B.mn_major, a.epilogue)) return cudaErrorInvalidValue;
+  }
+  const int nt = plan.nt;
   KernelFn kern = pick_kernel(a.A.mn_major, a.B.mn_major, a.epilogue, nt);
   if (!kern) return cudaErrorInvalidValue;
   const bool out_f32 = (a.epilogue == EPI_F32 || a.epilogue == EPI_F32_RESID);
@@ -825,10 +739,6 @@ cudaError_t gemm_launch(const GemmArgs& a, unsigned* err_word, int num_sms, cuda
   if (a.epilogue == EPI_DZ && (!a.targets || !a.lse)) return cudaErrorInvalidValue;
   if (a.rowscale && a.epilogue != EPI_F32) return cudaErrorInvalidValue;
   if (a.store_exp && (a.epilogue != EPI_LSE || !a.C)) return cudaErrorInvalidValue;
-
-  CUtensorMap tmA, tmB;
-  if (!encode_operand(&tmA, a.A, a.M, a.K, BM)) return cudaErrorInvalidValue;
-  if (!encode_operand(&tmB, a.B, a.N, a.K, BN / 2)) return cudaErrorInvalidValue;
 
   GemmDev p;
   p.M = a.M; p.N = a.N; p.K = a.K;
@@ -853,6 +763,10 @@ cudaError_t gemm_launch(const GemmArgs& a, unsigned* err_word, int num_sms, cuda
   p.tgt_logit = a.tgt_logit; p.lse = a.lse; p.scale = a.scale; p.col0 = a.col0;
   p.rowscale = a.rowscale; p.store_exp = a.store_exp;
   p.err = err_word;
+  if (plan.tn) return gemm_small_launch(a, p, plan.tn, plan.split, num_sms, stream);
+  CUtensorMap tmA, tmB;
+  if (!encode_gemm_operand(&tmA, a.A, a.M, a.K, BM)) return cudaErrorInvalidValue;
+  if (!encode_gemm_operand(&tmB, a.B, a.N, a.K, BN / 2)) return cudaErrorInvalidValue;
   const long long tiles = (long long)p.tiles_m * p.tiles_n * p.split_k;
   const int pairs = (int)(tiles < num_sms / 2 ? tiles : num_sms / 2);
   const int grid = 2 * pairs;

@@ -315,36 +315,24 @@ GemmArgs gemm_args(int M, int N, int K, const void* A, int lda, int a_mn, const 
   } while (0)
 
 // Weight-gradient GEMM dW[M,N] = dY^T X over K tokens.  The output has few tiles compared with the number of CTA
-// pairs, so the tile width (256 or 512 columns) and the number of work units per tile the token axis is split
-// into (partial sums are added atomically into the zeroed gradient) are chosen together, by a small model of
-// the kernel: waves of units over the pairs, times the k-slabs of a unit (a 512-wide slab costs 1.72 of a
-// 256-wide one) plus the unit's exposed prologue / epilogue.
+// pairs, so the kernel, its tile and the split of the token axis are chosen together (gemm_plan): partial sums are
+// added in a fixed order inside a cluster, or atomically into the zeroed gradient by units of the paired kernel.
 il_status wgrad(il_model* m, int k, int M, int N, int K, const bf16* dY, int ld_dy, const bf16* X, int ld_x, float* dW,
                 bool acc) {
-  const int pairs = m->sms[k] / 2;
-  const int slabs = (K + 63) / 64;
-  int best_nt = 1, best_s = 1;
-  double best_cost = 1e300;
-  for (int nt = 1; nt <= 2; ++nt) {
-    if (nt == 2 && N <= 256) break;
-    const int tiles = ((M + 255) / 256) * ((N + 256 * nt - 1) / (256 * nt));
-    const double slab_cost = nt == 1 ? 1.0 : 1.72, unit_cost = nt == 1 ? 2.0 : 10.0;
-    for (int s = 1; s <= 8; ++s) {
-      if (s > 1 && slabs / s < 16) break;
-      const int per = (slabs + s - 1) / s;
-      const int waves = (tiles * s + pairs - 1) / pairs;
-      const double cost = waves * (per * slab_cost + unit_cost) + (s > 1 ? 4.0 : 0.0);   // + zeroing the output
-      if (cost < best_cost * 0.97) { best_cost = cost; best_nt = nt; best_s = s; }
-    }
-  }
   GemmArgs g = gemm_args(M, N, K, dY, ld_dy, 1, X, ld_x, 1, EPI_F32, dW, N);
-  g.tile_blocks = best_nt;
-  if (best_s > 1) {
-    // split units add their partial sums into the output: zero it first, unless this pass adds to the last one's
-    if (!acc) IL_CUDA(m, cudaMemsetAsync(dW, 0, (size_t)M * N * sizeof(float), m->streams[k]));
-    g.split_k = best_s;
-  } else {
+  const GemmPlan plan = gemm_plan(M, N, K, 1, 1, EPI_F32, m->sms[k], 8);
+  if (plan.tn) {
+    g.tile_blocks = -((plan.tn == 64 ? 64 : 0) + plan.split);
     g.accumulate = acc ? 1 : 0;
+  } else {
+    g.tile_blocks = plan.nt;
+    if (plan.split_k > 1) {
+      // split units add their partial sums into the output: zero it first, unless this pass adds to the last one's
+      if (!acc) IL_CUDA(m, cudaMemsetAsync(dW, 0, (size_t)M * N * sizeof(float), m->streams[k]));
+      g.split_k = plan.split_k;
+    } else {
+      g.accumulate = acc ? 1 : 0;
+    }
   }
   return gemm(m, k, g);
 }
