@@ -521,6 +521,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     tc_fence_after();
     tmem_dealloc_pair(tmem_base, TMEM_COLS);
   }
+  // Freeing a pair's tensor memory concerns both SMs.  Without this second barrier one CTA could exit, and a CTA of
+  // another kernel (the dependent one, or another stream's) allocate on its SM, before the peer has freed its half.
+  __syncthreads();
+  cluster_sync_all();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -649,34 +653,45 @@ bool encode_gemm_operand(CUtensorMap* tm, const GemmOperand& op, int rows, int k
 }
 
 // Which kernel and tile, from a model of each one's time in microseconds.  The constants are measured (back-to-back
-// launches of the shapes of a training step from 256 to 16384 tokens, d 128 to 2560); the model is within about 15 % of
-// the measurements and the choice within 10 % of the best of all candidates on nearly all of them.
+// launches of the shapes of a training step from 256 to 16384 tokens, d 128 to 2560); the choice is within 10 % of the
+// best candidate on nearly all of them.
 //   paired, 256 x 256: 0.283 us per slab alone, 0.345 with all pairs busy; a wave costs its main loop or its epilogue,
 //     whichever is longer (the accumulators alternate).
-//   paired, 256 x 512: 0.55 / 0.64 per slab (of twice the columns), the epilogue is exposed.  Taken up to 10 % behind
-//     the square tile: it moves a quarter fewer operand bytes, which counts beside other streams and under the power cap.
-//   128 x 128 / 128 x 64: 0.26 / 0.245 per slab while each CTA has an SM to itself, 0.46 / 0.33 with two per SM.
+//   paired, 256 x 512: 0.55 / 0.64 per slab (of twice the columns), the epilogue is exposed; only for k-ranges of 2048
+//     and more (8192 x 4096 x 1024 with the saved derivative: 112 us against 73 with square tiles).  Counted at 0.86: it
+//     moves a quarter fewer operand bytes, which back-to-back launches of one shape do not show but the power cap does.
+//   128 x 128 / 128 x 64: 0.26 / 0.245 per slab while each CTA has an SM to itself, 0.46 / 0.33 with two per SM, then
+//     counted at 1.1 for the opposite reason (twice the operand bytes of the square tile).
 // max_atomic_split > 1 (EPI_F32 into a zeroed output): the paired kernel may split the contraction over up to that
 // many units that add with red.global.add; 3 us for the zeroing pass.
-GemmPlan gemm_plan(int M, int N, int K, int a_mn, int b_mn, int epi, int num_sms, int max_atomic_split) {
+// concurrency: how many streams run work like this at the same time.  A kernel that takes t on a fraction f of the
+// SMs costs such a set of streams max(t / concurrency, f t): alone, latency decides; beside others, SM time does.
+GemmPlan gemm_plan(int M, int N, int K, int a_mn, int b_mn, int epi, int num_sms, int max_atomic_split, int concurrency) {
   const int slabs = (K + BK - 1) / BK, pairs = num_sms / 2;
+  const float ic = 1.0f / (concurrency > 1 ? concurrency : 1);
   // epilogue of a 256 x 256 tile in steady state / exposed after the last tile, by epilogue
   static const float EPI_STEADY[EPI_COUNT] = {5.0f, 8.2f, 10.0f, 9.5f, 5.5f, 7.0f, 6.0f};
   static const float EPI_LAST[EPI_COUNT] = {0.8f, 3.2f, 3.2f, 4.2f, 3.0f, 2.0f, 2.0f};
   GemmPlan best{0, 1, 1, 1, 1e30f};
+  auto consider = [&](GemmPlan cand, float t, float fraction) {
+    cand.us = t * (fraction > ic ? fraction : ic);
+    if (cand.us < best.us * 0.98f) best = cand;
+  };
   for (int nt = 1; nt <= 2; ++nt) {
     if (nt == 2 && N <= BN) break;
     const int tiles = ((M + TILE_M - 1) / TILE_M) * ((N + nt * BN - 1) / (nt * BN));
     for (int s = 1; s <= (max_atomic_split > 1 ? max_atomic_split : 1); ++s) {
       if (s > 1 && slabs / s < 16) break;
       const int per = (slabs + s - 1) / s, units = tiles * s, waves = (units + pairs - 1) / pairs;
+      if (nt == 2 && per < 32) break;
       const float load = units < pairs ? (float)units / pairs : 1.0f;
       const float main = per * (nt == 1 ? 0.283f + 0.062f * load : 0.55f + 0.09f * load);
+      const float steady = EPI_STEADY[epi] * (s > 1 ? 1.6f : 1.0f);        // atomic adds instead of stores
       float t;
-      if (nt == 1) t = 4.5f + (waves - 1) * (main > EPI_STEADY[epi] ? main : EPI_STEADY[epi]) + main + EPI_LAST[epi];
-      else t = 0.9f * (4.5f + waves * (main + 1.1f * EPI_STEADY[epi]) + EPI_LAST[epi]);
+      if (nt == 1) t = 4.5f + (waves - 1) * (main > steady ? main : steady) + main + EPI_LAST[epi];
+      else t = 0.86f * (4.5f + waves * (main + 1.1f * EPI_STEADY[epi]) + EPI_LAST[epi]);
       if (s > 1) t += 3.0f;
-      if (t < best.us * 0.98f) best = GemmPlan{0, 1, nt, s, t};
+      consider(GemmPlan{0, 1, nt, s, 0.f}, t, (float)units / (waves * pairs));
     }
   }
   if (!gemm_small_supported(a_mn, b_mn, epi)) return best;
@@ -694,11 +709,12 @@ GemmPlan gemm_plan(int M, int N, int K, int a_mn, int b_mn, int epi, int num_sms
       float t = 3.2f + (s == 1 ? 0.f : s == 8 ? 3.0f : 2.0f);
       if (ctas <= room) {
         t += per * (tn == 64 ? 0.245f : 0.26f) + e;
+        consider(GemmPlan{tn, s, 1, 1, 0.f}, t, (float)ctas / room);
       } else {
         const int rounds = (int)((ctas + 2 * room - 1) / (2 * room));
         t += rounds * (per * (tn == 64 ? 0.33f : 0.46f) + e) + 1.0f + 3.0f * (rounds - 1);
+        consider(GemmPlan{tn, s, 1, 1, 0.f}, 1.1f * t, (float)ctas / (2.0f * room * rounds));
       }
-      if (t < best.us * 0.98f) best = GemmPlan{tn, s, 1, 1, t};
     }
   }
   return best;
@@ -709,7 +725,7 @@ cudaError_t gemm_launch(const GemmArgs& a, unsigned* err_word, int num_sms, cuda
   if (e != cudaSuccess) return e;
   if (a.M <= 0 || a.N <= 0 || a.K <= 0 || !a.A.ptr || !a.B.ptr || !err_word) return cudaErrorInvalidValue;
   if ((a.A.ld % 8) || (a.B.ld % 8) || ((uintptr_t)a.A.ptr % 16) || ((uintptr_t)a.B.ptr % 16)) return cudaErrorInvalidValue;
-  GemmPlan plan = gemm_plan(a.M, a.N, a.K, a.A.mn_major, a.B.mn_major, a.epilogue, num_sms, 0);
+  GemmPlan plan = gemm_plan(a.M, a.N, a.K, a.A.mn_major, a.B.mn_major, a.epilogue, num_sms, 0, a.concurrency);
   const bool atomic_split = a.split_k > 1 && a.epilogue == EPI_F32 && !a.accumulate;
   if (a.tile_blocks > 0 || atomic_split) {       // the paired kernel, as asked for
     plan.tn = 0;

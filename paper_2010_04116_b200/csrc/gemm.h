@@ -56,12 +56,14 @@ struct GemmArgs {
   int tile_blocks;    // 256-column blocks per output tile of a CTA pair: 1 (256 x 256), 2 (256 x 512); negative: tiles of one
                       // CTA, -S (128 x 128) or -(64 + S) (128 x 64) with the contraction split over a cluster of S = 1,
                       // 2, 4, 8 CTAs; 0 = chosen from the shape
+  int concurrency;    // streams that run work like this at the same time (0 = 1): weighs latency against SM time
 };
 
 // Kernel and tile for a shape: tn = 0: CTA pairs with nt 256-column blocks per tile and split_k atomically added
 // k-ranges; tn = 64 / 128: single-CTA tiles of that width, k split over a cluster of `split`.  us = modelled time.
 struct GemmPlan { int tn, split, nt, split_k; float us; };
-GemmPlan gemm_plan(int M, int N, int K, int a_mn, int b_mn, int epi, int num_sms, int max_atomic_split);
+GemmPlan gemm_plan(int M, int N, int K, int a_mn, int b_mn, int epi, int num_sms, int max_atomic_split,
+                   int concurrency);
 
 // Enqueue one GEMM on `stream`.  `err_word` is a device word set non-zero when a bounded wait in
 // the kernel expired.  Returns a cudaError_t (argument errors are reported as cudaErrorInvalidValue).

@@ -320,7 +320,7 @@ GemmArgs gemm_args(int M, int N, int K, const void* A, int lda, int a_mn, const 
 il_status wgrad(il_model* m, int k, int M, int N, int K, const bf16* dY, int ld_dy, const bf16* X, int ld_x, float* dW,
                 bool acc) {
   GemmArgs g = gemm_args(M, N, K, dY, ld_dy, 1, X, ld_x, 1, EPI_F32, dW, N);
-  const GemmPlan plan = gemm_plan(M, N, K, 1, 1, EPI_F32, m->sms[k], 8);
+  const GemmPlan plan = gemm_plan(M, N, K, 1, 1, EPI_F32, m->sms[k], 8, 1);
   if (plan.tn) {
     g.tile_blocks = -((plan.tn == 64 ? 64 : 0) + plan.split);
     g.accumulate = acc ? 1 : 0;
@@ -1099,12 +1099,16 @@ il_status head_backward(il_model* m, int k, bool acc, float scale) {
   const int N = m->ntok, d = m->d, V = m->V;
   const HeadOff& o = m->head_off[k];
   HeadScratch& h = m->hs[k];
+  // all heads' backward passes are enqueued at once, each on its own stream: dU, whose few output tiles leave most of
+  // the GPU idle on small batches, is planned as one of (at least) two that run side by side
+  const int beside = m->placement == IL_PLACE_SINGLE && m->K > 1 ? 2 : 1;
   if (m->head_mode == IL_HEAD_STORED) {
     IL_K(m, head_backward_prepare(h.z, m->ldz, h.lse, m->targets[k], h.u, h.us, h.rs, N, d, scale, m->err_word[k], st));
     {  // dU = diag(s) (E' W).  Not split over the contraction: atomically added partial sums would make dU, and
        // with it every gradient below this head, depend on the order the work units finish in.
       GemmArgs g = gemm_args(N, d, V, h.z, m->ldz, 0, m->Pb[k] + o.w, d, 1, EPI_F32, h.du, d);
       g.rowscale = h.rs;
+      g.concurrency = beside;
       IL_TRY(gemm(m, k, g));
     }
     {  // dW = E'^T (diag(s) U)
@@ -1131,6 +1135,7 @@ il_status head_backward(il_model* m, int k, bool acc, float scale) {
       {
         GemmArgs g = gemm_args(N, d, w, h.z, chunk, 0, m->Pb[k] + o.w + (size_t)c0 * d, d, 1, EPI_F32, h.du, d);
         g.accumulate = c0 > 0 ? 1 : 0;
+        g.concurrency = beside;
         IL_TRY(gemm(m, k, g));
       }
       {
