@@ -10,7 +10,9 @@ namespace il {
 // a_0[i,:] = wte[clamp(tok[i]),:] + wpe[i % T,:]  (fp32 residual stream)
 cudaError_t embed_fwd(const int* tok, const float* wte, const float* wpe, float* x, int ntok, int T, int d, int V,
                       cudaStream_t s);
-// keys [ntok rounded up to 8192] = the batch's (token, position) pairs in sorted order, for embed_bwd.  V < 2^19.
+// keys [embed_sort_words(ntok)] = the batch's (token, position) pairs in sorted order and the runs of equal tokens, for
+// embed_bwd.  V < 2^19.
+size_t embed_sort_words(size_t ntok);
 cudaError_t embed_sort(const int* tok, unsigned* keys, int ntok, int V, cudaStream_t s);
 // dwte[t,:] = (accumulate ? dwte[t,:] : 0) + sum over the positions i with tok[i] = t of dx[i,:], summed in position
 // order (deterministic; rows of tokens that do not occur are left as they are: zero them first unless accumulating);

@@ -98,7 +98,7 @@ struct il_model {
   // side stream that waits for that point only (ev_head), beside the component's backward.
   std::vector<cudaStream_t> side;
   std::vector<cudaEvent_t> ev_head, ev_side;
-  cudaEvent_t ev_batch;
+  cudaEvent_t ev_batch, ev_sort;      // the batch is on the device; its token keys are sorted
   // parameters
   std::vector<TensorRec> tensors;
   std::vector<LayerOff> layer_off;   // K*Lc main layers, then K*Lh head layers (head k's at K*Lc + k*Lh)
@@ -584,6 +584,7 @@ extern "C" il_status il_create(int K, int Lc, int d, int H, int F, int V, int n,
   }
   IL_CUDA(m, cudaSetDevice(m->dev[0]));
   IL_CUDA(m, cudaEventCreateWithFlags(&m->ev_batch, cudaEventDisableTiming));
+  IL_CUDA(m, cudaEventCreateWithFlags(&m->ev_sort, cudaEventDisableTiming));
 
   // ---- parameter, gradient and optimiser storage
   // All host<->device copies of the library are stream-ordered on the owning component's stream (a synchronous
@@ -696,7 +697,7 @@ extern "C" il_status il_create(int K, int Lc, int d, int H, int F, int V, int n,
     IL_CUDA(m, cudaMemsetAsync(m->losses[k], 0, K * 4, m->streams[k]));
   }
   IL_CUDA(m, cudaSetDevice(m->dev[0]));
-  IL_TRY(dev_alloc_t(m, &m->sort_keys[0], (N + 8191) / 8192 * 8192));     // embedding backward: sorted (token, position) keys
+  IL_TRY(dev_alloc_t(m, &m->sort_keys[0], embed_sort_words(N)));     // embedding backward: sorted (token, position) keys
   m->fwd_done.assign(K, 0);
   m->loss_done.assign(K, 0);
   for (int dv : m->dev_list) {
@@ -727,6 +728,7 @@ extern "C" il_status il_destroy(il_model* m) {
   for (auto e : m->ev_side) cudaEventDestroy(e);
   for (auto st : m->side) cudaStreamDestroy(st);
   if (m->ev_batch) cudaEventDestroy(m->ev_batch);
+  if (m->ev_sort) cudaEventDestroy(m->ev_sort);
   for (auto e : m->prof_pool) cudaEventDestroy(e);
   for (auto& r : m->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
   if (m->own_streams)
@@ -862,6 +864,7 @@ extern "C" il_status il_set_batch(il_model* m, const int* tokens, const int* tar
   IL_TRY(join_all(m));
   cudaStream_t s0 = m->streams[0];
   const size_t bytes = (size_t)B * T * sizeof(int);
+  IL_CUDA(m, cudaStreamWaitEvent(s0, m->ev_sort, 0));     // the last batch's ids have been read by the sort
   const cudaMemcpyKind kind = on_device ? cudaMemcpyDefault : cudaMemcpyHostToDevice;
   IL_CUDA(m, cudaEventRecord(m->ev_batch, s0));
   for (int k = 0; k < m->K; ++k) {
@@ -872,10 +875,13 @@ extern "C" il_status il_set_batch(il_model* m, const int* tokens, const int* tar
     IL_CUDA(m, cudaMemcpyAsync(m->targets[k], targets, bytes, kind, m->streams[k]));
   }
   IL_CUDA(m, cudaSetDevice(m->dev[0]));
-  // (token, position) keys in sorted order for the embedding backward: known as soon as the batch is
-  IL_K(m, embed_sort(m->tokens[0], m->sort_keys[0], B * T, m->V, s0));
+  // (token, position) keys in sorted order for the embedding backward: made on component 0's side stream beside the
+  // forward pass (44 us for 8192 positions, which would otherwise precede every step's first kernel)
+  IL_CUDA(m, cudaEventRecord(m->ev_batch, s0));
+  IL_CUDA(m, cudaStreamWaitEvent(m->side[0], m->ev_batch, 0));
+  IL_K(m, embed_sort(m->tokens[0], m->sort_keys[0], B * T, m->V, m->side[0]));
+  IL_CUDA(m, cudaEventRecord(m->ev_sort, m->side[0]));
   if (m->tokens[1 % m->K] == m->tokens[0]) {     // shared buffers: the other streams start after the copies
-    IL_CUDA(m, cudaEventRecord(m->ev_batch, s0));
     for (int k = 1; k < m->K; ++k) IL_CUDA(m, cudaStreamWaitEvent(m->streams[k], m->ev_batch, 0));
   }
   m->B = B; m->T = T; m->ntok = B * T;
@@ -1244,6 +1250,7 @@ extern "C" il_status il_backward_nwise(il_model* m) {
         IL_TRY(component_backward(m, k, s, acc));
       }
       if (k == 0) {
+        IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_sort, 0));
         IL_K(m, embed_bwd(m->tokens[k], m->sort_keys[0], m->cs[0].dx, m->G[k] + m->off_wte, m->G[k] + m->off_wpe, N, m->T, d, m->V, acc ? 1 : 0, st));
         m->launches++;
       }
@@ -1307,6 +1314,7 @@ extern "C" il_status il_backward_nwise(il_model* m) {
         IL_TRY(component_backward(m, k, used, acc));
       }
       if (k == 0) {
+        IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_sort, 0));
         IL_K(m, embed_bwd(m->tokens[k], m->sort_keys[0], m->cs[0].dx, m->G[k] + m->off_wte, m->G[k] + m->off_wpe, N, m->T, d, m->V, acc ? 1 : 0, st));
         m->launches++;
       }
