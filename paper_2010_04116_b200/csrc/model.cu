@@ -60,6 +60,18 @@ struct HeadScratch {
   float* rs; // [Ntok]: exp(-lse) / Ntok (stored mode)
 };
 
+// A stretch of one component stream's work that depends on nothing but the model's own buffers and a few integers (the
+// key), recorded as a CUDA graph when it is asked for a second time and replayed from then on.
+struct Segment {
+  int kind, k;
+  int key[6];
+  int uses;                            // -1: could not be recorded, always enqueued directly
+  long long launches, stamp;
+  cudaGraphExec_t exec;
+};
+enum { SEG_FORWARD, SEG_HEAD_LOSS, SEG_HEAD_BACKWARD, SEG_COMPONENT_BACKWARD };
+constexpr size_t SEGMENTS_PER_STREAM = 16;     // four kinds, a few batch shapes each; the least recently used one goes
+
 struct ProfRec { cudaEvent_t a, b; double flops; };
 
 // Named range on the host timeline of a profiler (NVTX; costs nothing when no tool is attached): one per call of
@@ -144,6 +156,8 @@ struct il_model {
   // profiling
   int prof;                           // 0 off, 1 events around each GEMM, 2 the same with the GEMM alone on the GPU
   std::vector<ProfRec> prof_recs;
+  std::vector<std::vector<Segment>> segments;   // per component
+  long long segment_clock;
   std::vector<cudaEvent_t> prof_pool;
   std::string err;
 };
@@ -341,6 +355,11 @@ il_status alloc_scratch(il_model* m, int s_cap) {
   // Backward scratch for s_cap stacked gradient streams per component.  It only grows; a superseded set is handed
   // back before the larger one is obtained (the callers have synchronised the devices).
   if (s_cap <= m->s_cap) return IL_OK;
+  for (auto& v : m->segments) {            // recordings refer to the scratch that is about to go
+    for (Segment& s : v)
+      if (s.exec) cudaGraphExecDestroy(s.exec);
+    v.clear();
+  }
   const size_t R = (size_t)s_cap * m->ntok_max;
   const int d = m->d, F = m->F;
   for (auto& c : m->cs) {
@@ -441,7 +460,7 @@ extern "C" il_status il_create(int K, int Lc, int d, int H, int F, int V, int n,
   m->max_batch = opt->max_batch; m->max_seq = opt->max_seq;
   m->ntok_max = opt->max_batch * opt->max_seq;
   m->ln_eps = opt->ln_eps > 0 ? opt->ln_eps : 1e-5f;
-  m->rule = IL_RULE_SUM; m->step = 0; m->adamw_issued = 0; m->bytes = 0; m->launches = 0; m->s_cap = 0;
+  m->rule = IL_RULE_SUM; m->step = 0; m->adamw_issued = 0; m->segment_clock = 0; m->segments.resize((size_t)K); m->bytes = 0; m->launches = 0; m->s_cap = 0;
   m->prof = 0; m->batch_set = false; m->bwd_done = false;
   m->B = m->T = m->ntok = 0;
   m->ev_batch = nullptr;
@@ -715,6 +734,9 @@ extern "C" il_status il_destroy(il_model* m) {
     cudaSetDevice(dv);
     cudaDeviceSynchronize();
   }
+  for (auto& v : m->segments)
+    for (Segment& s : v)
+      if (s.exec) cudaGraphExecDestroy(s.exec);
   for (auto& pr : m->allocs) {
     cudaSetDevice(pr.second);
     if (m->opt.free_) m->opt.free_(pr.first, m->opt.alloc_ctx);
@@ -896,6 +918,69 @@ extern "C" il_status il_set_batch(il_model* m, const int* tokens, const int* tar
 
 namespace {
 
+// Enqueue `body` (work on component k's stream only: kernels, memsets and copies between the model's own buffers, no
+// events) directly the first time, and as a recorded graph from the second time on.  A tiny step is ~100 kernels of
+// 2-4 us; enqueued one by one each costs the host about 4 us (tensor maps, launch attributes), a graph of them 5-10 us
+// in all.  Nothing in a recording refers to a caller's buffer: the batch is copied into the model's own memory first.
+template <class F>
+il_status run_segment(il_model* m, int kind, int k, const int (&key)[6], F&& body) {
+  cudaStream_t st = m->streams[k];
+  if (m->prof) return body();                    // (timing of single GEMMs needs their events)
+  Segment* s = nullptr;
+  for (Segment& c : m->segments[k])
+    if (c.kind == kind && memcmp(c.key, key, sizeof key) == 0) { s = &c; break; }
+  if (!s) {
+    std::vector<Segment>& v = m->segments[k];
+    if (v.size() >= SEGMENTS_PER_STREAM) {
+      size_t old = 0;
+      for (size_t i = 1; i < v.size(); ++i)
+        if (v[i].stamp < v[old].stamp) old = i;
+      if (v[old].exec) {
+        IL_CUDA(m, cudaStreamSynchronize(st));                 // its last launch may still be running
+        cudaGraphExecDestroy(v[old].exec);
+      }
+      v.erase(v.begin() + (long)old);
+    }
+    Segment n;
+    memset(&n, 0, sizeof n);
+    n.kind = kind; n.k = k;
+    memcpy(n.key, key, sizeof key);
+    v.push_back(n);
+    s = &v.back();
+  }
+  s->stamp = ++m->segment_clock;
+  if (!s->exec) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (s->uses < 1 || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      if (s->uses >= 0) s->uses++;
+      return body();
+    }
+    const long long l0 = m->launches;
+    if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+      cudaGetLastError();
+      s->uses = -1;
+      return body();
+    }
+    const il_status rs = body();
+    cudaGraph_t g = nullptr;
+    const cudaError_t e = cudaStreamEndCapture(st, &g);
+    s->launches = m->launches - l0;
+    m->launches = l0;
+    cudaGraphExec_t exec = nullptr;
+    if (rs != IL_OK || e != cudaSuccess || !g || cudaGraphInstantiate(&exec, g, 0) != cudaSuccess) {
+      cudaGetLastError();
+      if (g) cudaGraphDestroy(g);
+      s->uses = -1;
+      return body();
+    }
+    cudaGraphDestroy(g);
+    s->exec = exec;
+  }
+  IL_CUDA(m, cudaGraphLaunch(s->exec, st));
+  m->launches += s->launches;
+  return IL_OK;
+}
+
 // `count` consecutive pre-LN blocks (layer records base .. base+count-1) applied to x_in on stream k.
 il_status layers_forward(il_model* m, int k, size_t base, int count, const float* x_in) {
   cudaStream_t st = m->streams[k];
@@ -947,9 +1032,7 @@ extern "C" il_status il_forward_component(il_model* m, int k) {
   IL_CUDA(m, cudaSetDevice(m->dev[k]));
   cudaStream_t st = m->streams[k];
   const int N = m->ntok, d = m->d;
-  if (k == 0) {
-    IL_K(m, embed_fwd(m->tokens[k], m->P[k] + m->off_wte, m->P[k] + m->off_wpe, m->a[0], N, m->T, d, m->V, st));
-  } else {
+  if (k > 0) {
     IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_fwd[k - 1], 0));
     // pipeline placement (Sec. 3: the module's output is sent to the next accelerator): a_k is copied into a
     // buffer this component's device owns; every kernel of the component then reads local memory only
@@ -958,7 +1041,13 @@ extern "C" il_status il_forward_component(il_model* m, int k) {
       m->xfer_log.push_back(0); m->xfer_log.push_back(k - 1); m->xfer_log.push_back(-1);
     }
   }
-  IL_TRY(layers_forward(m, k, (size_t)k * m->Lc, m->Lc, comp_input(m, k)));
+  {
+    const int key[6] = {m->B, m->T, 0, 0, 0, 0};
+    IL_TRY(run_segment(m, SEG_FORWARD, k, key, [&]() -> il_status {
+      if (k == 0) IL_K(m, embed_fwd(m->tokens[k], m->P[k] + m->off_wte, m->P[k] + m->off_wpe, m->a[0], N, m->T, d, m->V, st));
+      return layers_forward(m, k, (size_t)k * m->Lc, m->Lc, comp_input(m, k));
+    }));
+  }
   IL_CUDA(m, cudaEventRecord(m->ev_fwd[k], st));
   m->fwd_done[k] = 1;
   return IL_OK;
@@ -974,6 +1063,8 @@ extern "C" il_status il_aux_head_loss(il_model* m, int k, float* loss_host) {
   IL_CUDA(m, cudaSetDevice(m->dev[k]));
   cudaStream_t st = m->streams[k];
   if (!m->loss_done[k]) {
+    const int key[6] = {m->B, m->T, m->head_mode, 0, 0, 0};
+    IL_TRY(run_segment(m, SEG_HEAD_LOSS, k, key, [&]() -> il_status {
     const int N = m->ntok, d = m->d, V = m->V;
     const HeadOff& o = m->head_off[k];
     HeadScratch& h = m->hs[k];
@@ -995,6 +1086,8 @@ extern "C" il_status il_aux_head_loss(il_model* m, int k, float* loss_host) {
     // per-row log-sum-exp and negative log-likelihood, then the mean of the latter in a fixed summation order
     IL_K(m, lse_finalize(h.pmax, h.psum, m->part_ld, m->part_ld, h.tgt_logit, h.lse, h.nll, N, st));
     IL_K(m, mean_f32(h.nll, N, m->losses[k] + k, st));
+    return IL_OK;
+    }));
     m->loss_done[k] = 1;
   }
   if (loss_host) {
@@ -1165,7 +1258,10 @@ il_status head_backward(il_model* m, int k, bool acc, float scale) {
 }
 
 il_status component_backward(il_model* m, int k, int s, bool acc) {
-  return layers_backward(m, k, s, (size_t)k * m->Lc, m->Lc, comp_input(m, k), acc);
+  const int key[6] = {m->B, m->T, s, acc ? 1 : 0, 0, 0};
+  return run_segment(m, SEG_COMPONENT_BACKWARD, k, key, [&]() -> il_status {
+    return layers_backward(m, k, s, (size_t)k * m->Lc, m->Lc, comp_input(m, k), acc);
+  });
 }
 
 }  // namespace
@@ -1219,7 +1315,8 @@ extern "C" il_status il_backward_nwise(il_model* m) {
     }
     {
       Range r2("head backward %d", k);
-      IL_TRY(head_backward(m, k, acc, gscale));
+      const int key[6] = {m->B, m->T, m->head_mode, acc ? 1 : 0, m->micro, 0};
+      IL_TRY(run_segment(m, SEG_HEAD_BACKWARD, k, key, [&]() -> il_status { return head_backward(m, k, acc, gscale); }));
     }
     IL_CUDA(m, cudaEventRecord(m->ev_head[k], st));      // head k's parameter gradients are final from here on
   }

@@ -1,0 +1,62 @@
+"""The parts of a step that are replayed as recorded graphs from their second use on give the bits of the first use."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+from paper_2010_04116_b200 import Model  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _model(rng, K=3, n=2, Lh=0, **kw):
+    m = Model(K, 1, 128, 4, 512, 300, n, 4, 48, head_layers=Lh, attn_bwd="two_kernels", **kw)
+    for name in m.names:
+        m.set_param(name, (rng.standard_normal(m.shapes[name]) * 0.05 + (1.0 if name.endswith(".g") else 0.0)).astype(np.float32))
+    return m
+
+
+def _batch(rng, B, T):
+    return tuple(rng.integers(0, 300, size=(B, T)).astype(np.int32) for _ in range(2))
+
+
+def _result(m, batch):
+    m.train_step(*batch)
+    losses = m.get_losses()
+    m.sync()
+    # weight matrices: sums of fixed order (vectors are summed atomically)
+    return [losses] + [m.get_grad(name) for name in m.names if len(m.shapes[name]) == 2]
+
+
+@pytest.mark.parametrize("kw", [{}, {"Lh": 1}, {"head_mode": "recompute"}, {"n": 1}])
+def test_replay_equals_first_use_for_each_shape(kw):
+    rng = np.random.default_rng(3)
+    m = _model(rng, **kw)
+    shapes = [(4, 48), (1, 48), (3, 31), (2, 1), (4, 17), (1, 7)]       # more than one stream's recordings hold
+    batches = [_batch(rng, *s) for s in shapes]
+    first = [_result(m, b) for b in batches]
+    l0 = m.stats()[1]
+    _result(m, batches[0])
+    per_step = m.stats()[1] - l0
+    for _ in range(3):
+        for f, b in zip(first, batches):
+            for x, y in zip(f, _result(m, b)):
+                assert np.array_equal(x, y)
+    l0 = m.stats()[1]
+    _result(m, batches[0])
+    assert m.stats()[1] - l0 == per_step                  # a replayed kernel counts like an enqueued one
+
+
+def test_replay_after_the_rule_and_window_change():
+    rng = np.random.default_rng(4)
+    m = _model(rng, K=4, n=1)
+    b = _batch(rng, 4, 48)
+    seen = {}
+    for n, rule in [(1, "sum"), (3, "sum"), (3, "mean"), (2, "far"), (1, "sum"), (3, "mean")] * 2:
+        m.set_n(n)
+        m.set_rule(rule)
+        for _ in range(3):
+            r = _result(m, b)
+            if (n, rule) in seen:
+                for x, y in zip(seen[n, rule], r):
+                    assert np.array_equal(x, y)
+            seen.setdefault((n, rule), r)
