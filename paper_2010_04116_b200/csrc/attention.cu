@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  grid_dep_sync();
+  grid_dep_wait();
   const uint32_t tmem_base = tmem_base_smem;                  // scores at columns [0, 64) (then P packed in [0, 32)), O at [64, 64 + dh)
   const uint32_t t_lane = tmem_base + ((uint32_t)(warp * 32) << 16);
   volatile int* abortp = &abort_flag;
@@ -223,6 +223,7 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(const __grid_constant_
       else umma_commit(bar_o);
     }
   }
+  grid_dep_launch();
   if (!fail && nkv > 0) {
     if (!mbar_wait(bar_o, 0, abortp)) { fail = 1; abort_flag = 1; }
     tc_fence_after();
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_const
   }
   tc_fence_before();
   __syncthreads();          // tensor memory is held by this CTA before the next kernel may become resident
-  grid_dep_sync();
+  grid_dep_wait();
   // lse (in log2 units) and delta of a query block: fetched from global memory into a register one sweep
   // step before they are put into shared memory (buffer j&1), two steps before they are used, so that no
   // step waits on that load
@@ -539,6 +540,7 @@ __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_const
     }
   }
   const int nit = nq - q0;
+  grid_dep_launch();
   if (!fail && nit > 0) {
     if (!mbar_wait(bar_acc, C::AHEAD ? 0u : ((uint32_t)(nit - 1) & 1u), abortp)) { fail = 1; abort_flag = 1; }
     tc_fence_after();
@@ -646,7 +648,7 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  grid_dep_sync();
+  grid_dep_wait();
   const uint32_t tmem_base = tmem_base_smem;     // S [0,64), dP [64,128) (later in part the packed dS), dQ [128,128+dh)
   const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
   volatile int* abortp = &abort_flag;
@@ -750,6 +752,7 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
       else umma_commit(bar_acc);
     }
   }
+  grid_dep_launch();
   if (!fail && nkv > 0) {
     if (!mbar_wait(bar_acc, C::AHEAD ? 0u : ((uint32_t)(nkv - 1) & 1u), abortp)) { fail = 1; abort_flag = 1; }
     tc_fence_after();
@@ -922,7 +925,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  grid_dep_sync();
+  grid_dep_wait();
   const uint32_t tmem_base = tmem_base_smem;
   const float c2 = scale * IL_LOG2E;
   int fail = 0;
@@ -972,6 +975,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
       }
       g += w.nit;
     }
+    grid_dep_launch();
   } else if (warp == 20 || warp == 21) {
     // ---------------------------------------------------------------- MMA issue, one thread per half x of the query block
     // A thread issues small MMAs no faster than one per ~54 cycles, and every hand-over between threads costs a
@@ -1266,7 +1270,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
 // dqkv[row, h*dh + c] (the Q third) = bf16(scale * dq_acc[row, h*dh + c]): the accumulated dQ leaves fp32 here.
 __global__ void __launch_bounds__(256) attn_dq_convert_kernel(const float* __restrict__ acc, bf16* __restrict__ dqkv, size_t rows,
                                                               int d, float scale) {
-  grid_dep_sync();
+  grid_dep_wait();
   const int d8 = d >> 3;
   const size_t total = rows * (size_t)d8;
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < total; i += (size_t)gridDim.x * 256) {
@@ -1291,7 +1295,7 @@ template <int DH>
 __global__ void __launch_bounds__(256) attn_delta_tc_kernel(const bf16* __restrict__ dout, const bf16* __restrict__ o,
                                                             float* __restrict__ delta, float* __restrict__ dq_zero, int NB,
                                                             int B, int T, int H) {
-  grid_dep_sync();
+  grid_dep_wait();
   constexpr int TPR = (DH == 80) ? 16 : DH / 8;      // threads per (row, head): a power of two (dh 80: 10 of 16 active)
   const long long gid = (long long)blockIdx.x * 256 + threadIdx.x;
   const long long item = gid / TPR;                  // (row, head) index
@@ -1322,6 +1326,7 @@ __global__ void __launch_bounds__(256) attn_delta_tc_kernel(const bf16* __restri
       }
     }
   }
+  grid_dep_launch();
 #pragma unroll
   for (int off = TPR / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
   if (item < total && part == 0) {

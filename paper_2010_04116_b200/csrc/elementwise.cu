@@ -13,7 +13,7 @@ static inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) 
 // ---------------------------------------------------------------------------------------------
 __global__ void embed_fwd_kernel(const int* __restrict__ tok, const float* __restrict__ wte,
                                  const float* __restrict__ wpe, float* __restrict__ x, int ntok, int T, int d, int V) {
-  grid_dep_sync();
+  grid_dep_wait();
   const int d4 = d >> 2;
   const size_t total = (size_t)ntok * d4;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
@@ -53,7 +53,7 @@ constexpr int SORT_STRIDE = 3 * SORT_CHUNK + 2;      // words per chunk: keys, (
 
 __global__ void __launch_bounds__(1024) embed_sort_kernel(const int* __restrict__ tok, unsigned* __restrict__ out, int ntok,
                                                           int V) {
-  grid_dep_sync();
+  grid_dep_wait();
   __shared__ unsigned sk[SORT_CHUNK];
   __shared__ int n_short, n_long;
   const int base = blockIdx.x * SORT_CHUNK;
@@ -117,7 +117,7 @@ cudaError_t embed_sort(const int* tok, unsigned* keys, int ntok, int V, cudaStre
 // 8192 x 1024 took 150-166 us, now 20.
 __global__ void __launch_bounds__(256) embed_bwd_wte_kernel(const unsigned* __restrict__ sorted, const float* __restrict__ dx,
                                                             float* __restrict__ dwte, int d, int accumulate) {
-  grid_dep_sync();
+  grid_dep_wait();
   __shared__ float4 part[8][32];
   constexpr unsigned POS_MASK = (1u << SORT_POS_BITS) - 1u;
   const unsigned* keys = sorted;
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256) embed_bwd_wte_kernel(const unsigned* __re
 }
 __global__ void embed_bwd_wpe_kernel(const float* __restrict__ dx, float* __restrict__ dwpe, int B, int T, int d,
                                      int accumulate) {
-  grid_dep_sync();
+  grid_dep_wait();
   const int d4 = d >> 2;
   const size_t total = (size_t)T * d4;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(256) layernorm_fwd_kernel(const float* __restr
                                                             const float* __restrict__ beta, bf16* __restrict__ y,
                                                             float* __restrict__ mean, float* __restrict__ rstd,
                                                             int rows, int d, float eps) {
-  grid_dep_sync();
+  grid_dep_wait();
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(256) layernorm_fwd_kernel(const float* __restr
     const float a = v.x - mu, b = v.y - mu, cc = v.z - mu, e = v.w - mu;
     q += (a * a + b * b) + (cc * cc + e * e);
   }
+  grid_dep_launch();
   const float rs = rsqrtf(warp_sum(q) / d + eps);
   if (lane == 0) { mean[row] = mu; rstd[row] = rs; }
   uint2* yr = reinterpret_cast<uint2*>(y + (size_t)row * d);
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(256) layernorm_fwd_reg_kernel(const float* __r
                                                                 const float* __restrict__ beta, bf16* __restrict__ y,
                                                                 float* __restrict__ mean, float* __restrict__ rstd,
                                                                 int rows, float eps) {
-  grid_dep_sync();
+  grid_dep_wait();
   constexpr int d = NV * 128;
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -261,6 +262,7 @@ __global__ void __launch_bounds__(256) layernorm_fwd_reg_kernel(const float* __r
     v[i].x -= mu; v[i].y -= mu; v[i].z -= mu; v[i].w -= mu;
     q += (v[i].x * v[i].x + v[i].y * v[i].y) + (v[i].z * v[i].z + v[i].w * v[i].w);
   }
+  grid_dep_launch();
   const float rs = rsqrtf(warp_sum(q) / d + eps);
   if (lane == 0) { mean[row] = mu; rstd[row] = rs; }
   uint2* yr = reinterpret_cast<uint2*>(y + (size_t)row * d);
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(256) layernorm_bwd_rows_kernel(const void* __r
                                                                  const float* __restrict__ gamma, const float* resid,
                                                                  float* dx_out, bf16* __restrict__ dx_bf16, int rows,
                                                                  int x_rows, int d) {
-  grid_dep_sync();
+  grid_dep_wait();
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -330,6 +332,7 @@ __global__ void __launch_bounds__(256) layernorm_bwd_rows_kernel(const void* __r
   }
   const float m1 = warp_sum(s1) / d;
   const float m2 = warp_sum(s2) * rs / d;   // mean of dxhat * xhat
+  grid_dep_launch();
   const float4* rr = resid ? reinterpret_cast<const float4*>(resid + (size_t)row * d) : nullptr;
   float4* outr = reinterpret_cast<float4*>(dx_out + (size_t)row * d);
   uint2* outb = dx_bf16 ? reinterpret_cast<uint2*>(dx_bf16 + (size_t)row * d) : nullptr;
@@ -385,7 +388,7 @@ __global__ void __launch_bounds__(256, 1) layernorm_bwd_fused_kernel(const bf16*
                                                                      float* dx_out, bf16* __restrict__ dx_bf16,
                                                                      float* __restrict__ dgamma, float* __restrict__ dbeta,
                                                                      float* __restrict__ colsum, int rows, int x_rows) {
-  grid_dep_sync();
+  grid_dep_wait();
   constexpr int d = NV * 128;
   __shared__ float4 red[8][NV * 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -447,6 +450,7 @@ __global__ void __launch_bounds__(256, 1) layernorm_bwd_fused_kernel(const bf16*
       if (first) { ac[i].x += o.x; ac[i].y += o.y; ac[i].z += o.z; ac[i].w += o.w; }
     }
   }
+  grid_dep_launch();
   // block-level combination, one quantity after the other through the same buffer
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
@@ -500,7 +504,7 @@ __global__ void __launch_bounds__(256) layernorm_bwd_params_kernel(const void* _
                                                                    const float* __restrict__ rstd,
                                                                    float* __restrict__ dgamma, float* __restrict__ dbeta,
                                                                    int rows, int d, int rows_per_block) {
-  grid_dep_sync();
+  grid_dep_wait();
   __shared__ float4 sg[8][32], sb[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c4 = blockIdx.x * 32 + lane;       // float4 column index
@@ -518,6 +522,7 @@ __global__ void __launch_bounds__(256) layernorm_bwd_params_kernel(const void* _
       ab.x += dv.x; ab.y += dv.y; ab.z += dv.z; ab.w += dv.w;
     }
   }
+  grid_dep_launch();
   sg[w][lane] = ag;
   sb[w][lane] = ab;
   __syncthreads();
@@ -559,7 +564,7 @@ cudaError_t layernorm_bwd_params(const void* dy, int dy_is_f32, const float* x, 
 template <bool IN_F32>
 __global__ void __launch_bounds__(256) colsum_kernel(const void* __restrict__ y, int ld, float* __restrict__ out, int rows,
                                                      int cols, int rows_per_block) {
-  grid_dep_sync();
+  grid_dep_wait();
   __shared__ float4 sm[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int c4 = blockIdx.x * 32 + lane;
@@ -580,6 +585,7 @@ __global__ void __launch_bounds__(256) colsum_kernel(const void* __restrict__ y,
       a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
     }
   }
+  grid_dep_launch();
   sm[w][lane] = a;
   __syncthreads();
   if (w == 0 && col_ok) {
@@ -612,7 +618,7 @@ cudaError_t colsum_f32(const float* y, int ld, float* out, int rows, int cols, c
 // ---------------------------------------------------------------------------------------------
 __global__ void add_convert_kernel(const float4* __restrict__ a, const float4* __restrict__ b, float4* out_f32,
                                    uint2* __restrict__ out_bf16, size_t n4) {
-  grid_dep_sync();
+  grid_dep_wait();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
     float4 v = a[i];
     if (b) {
@@ -642,7 +648,7 @@ cudaError_t add_convert(const float* a, const float* b, float* out_f32, bf16* ou
 struct LinComb { const float4* x[4]; float w[4]; int count; int accumulate; };
 
 __global__ void lincomb_convert_kernel(LinComb c, float4* out_f32, uint2* __restrict__ out_bf16, size_t n4) {
-  grid_dep_sync();
+  grid_dep_wait();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
     float4 v = c.accumulate ? out_f32[i] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -689,7 +695,7 @@ cudaError_t f32_to_bf16(const float* in, bf16* out, size_t n, cudaStream_t s) {
 __global__ void __launch_bounds__(256) lse_finalize_kernel(const float* __restrict__ pm, const float* __restrict__ ps,
                                                            int part_ld, int ntiles, const float* __restrict__ tgt_logit,
                                                            float* __restrict__ lse, float* __restrict__ nll, int rows) {
-  grid_dep_sync();
+  grid_dep_wait();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int row = blockIdx.x * 8 + w;
   if (row >= rows) return;
@@ -701,6 +707,7 @@ __global__ void __launch_bounds__(256) lse_finalize_kernel(const float* __restri
     const float tm = pm[(size_t)row * part_ld + t];
     if (tm > -INFINITY) sum += ps[(size_t)row * part_ld + t] * __expf(tm - m);
   }
+  grid_dep_launch();
   sum = warp_sum(sum);
   const float l = m + logf(sum);
   if (lane == 0) {
@@ -718,10 +725,11 @@ cudaError_t lse_finalize(const float* part_max, const float* part_sum, int part_
 // out[0] = mean of x[0..n) with a fixed summation order (one block: strided per-thread sums, then a tree), so the
 // value does not depend on scheduling.
 __global__ void __launch_bounds__(1024) mean_f32_kernel(const float* __restrict__ x, int n, float* __restrict__ out) {
-  grid_dep_sync();
+  grid_dep_wait();
   __shared__ float sm[1024];
   float a = 0.f;
   for (int i = threadIdx.x; i < n; i += 1024) a += x[i];
+  grid_dep_launch();
   sm[threadIdx.x] = a;
   __syncthreads();
   for (int o = 512; o > 0; o >>= 1) {
@@ -749,7 +757,7 @@ __global__ void __launch_bounds__(256) head_backward_prepare_kernel(bf16* __rest
                                                                     const int* __restrict__ targets, const bf16* __restrict__ u,
                                                                     bf16* __restrict__ u_scaled, float* __restrict__ rowscale,
                                                                     int rows, int d, float inv_rows, unsigned* err) {
-  grid_dep_sync();
+  grid_dep_wait();
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (row >= rows) return;
@@ -759,6 +767,7 @@ __global__ void __launch_bounds__(256) head_backward_prepare_kernel(bf16* __rest
     return;
   }
   const float s = __expf(-l) * inv_rows;
+  grid_dep_launch();
   if (lane == 0) {
     rowscale[row] = s;
     bf16* et = e + (size_t)row * ld + targets[row];
@@ -794,7 +803,7 @@ __global__ void __launch_bounds__(256) adamw_kernel(float4* __restrict__ p, floa
                                                     size_t n4_decay, float lr, float b1, float b2, float eps, float wd,
                                                     float ibc1, float ibc2, const unsigned* __restrict__ err,
                                                     unsigned* applied, size_t skip0, size_t skip1) {
-  grid_dep_sync();
+  grid_dep_wait();
   // a step whose kernels reported an error must not reach the parameters: leave everything as it is
   if (err && *reinterpret_cast<const volatile unsigned*>(err) != 0u) return;
   if (applied && blockIdx.x == 0 && threadIdx.x == 0) *applied += 1u;
@@ -837,7 +846,7 @@ cudaError_t adamw(float* p, float* m, float* v, const float* g, bf16* p_bf16, si
 // without any kernel having to go wrong.
 // ---------------------------------------------------------------------------------------------
 __global__ void wait_probe_kernel(unsigned* err, unsigned long long limit_ns) {
-  grid_dep_sync();
+  grid_dep_wait();
   __shared__ unsigned long long bar;
   __shared__ int never;
   if (threadIdx.x == 0) {

@@ -168,7 +168,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   __syncthreads();
   cluster_sync_all();       // the peer's barriers are initialised before anything is signalled remotely
   tc_fence_after();
-  grid_dep_sync();          // tensor memory is held, nothing in global memory has been touched yet
+  grid_dep_wait();          // tensor memory is held, nothing in global memory has been touched yet
   const uint32_t tmem_base = tmem_base_smem;
   volatile int* abortp = &abort_flag;
 
@@ -215,6 +215,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
+      grid_dep_launch();      // everything has been requested: the next kernel may set itself up on the SMs that become free
       if (!ok) {
         atomicExch(p.err, DEV_TIMEOUT_PRODUCER);
         abort_flag = 1;
@@ -691,7 +692,7 @@ GemmPlan gemm_plan(int M, int N, int K, int a_mn, int b_mn, int epi, int num_sms
       if (nt == 1) t = 4.5f + (waves - 1) * (main > steady ? main : steady) + main + EPI_LAST[epi];
       else t = 0.86f * (4.5f + waves * (main + 1.1f * EPI_STEADY[epi]) + EPI_LAST[epi]);
       if (s > 1) t += 3.0f;
-      consider(GemmPlan{0, 1, nt, s, 0.f}, t, (float)units / (waves * pairs));
+      consider(GemmPlan{0, 1, nt, s, 0.f}, t, waves > 1 ? 1.0f : load);       // (a static tile list: the last wave's idle pairs stay idle)
     }
   }
   if (!gemm_small_supported(a_mn, b_mn, epi)) return best;

@@ -91,7 +91,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  grid_dep_sync();          // tensor memory is held, nothing in global memory has been touched yet
+  grid_dep_wait();          // tensor memory is held, nothing in global memory has been touched yet
   const uint32_t tmem_base = tmem_base_smem;
   volatile int* abortp = &abort_flag;
 
@@ -154,6 +154,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
         if (++stage == stages) { stage = 0; phase ^= 1u; }
       }
+      grid_dep_launch();
     }
     __syncwarp();
     load_extra(0);
