@@ -276,6 +276,345 @@ __global__ void __launch_bounds__(128) attn_fwd_tc_kernel(const __grid_constant_
   }
 }
 
+// ------------------------------------------------------------------------------------------------
+// Forward for head dimensions up to 128: two query tiles in flight per SM.
+// One persistent CTA per SM walks (256 query rows, sequence, head) items, the long ones first, in snake order.  An item
+// is two 128-row tiles over the same key / value blocks of 128; tensor memory holds S (128 columns) and O (dh) of both.
+//   warps 0-3 / 4-7   softmax of tile 0 / 1, one thread per row, in halves of 64 keys: tcgen05.ld the scores, reference
+//                     maximum as above, P packed over the score columns; at the end of an item O / l to global memory
+//   warps 8, 9        one thread per tile issues the MMAs: P V of a half, then the next block's Q K^T of that half behind it (in
+//                     pipe order, so the score columns that hold P are free by then).  A tile's other half is in the
+//                     softmax threads' hands meanwhile, so they find their next scores ready
+//   warp 10           TMA: Q of an item, a ring of K and one of V
+// While one tile's softmax runs, the pipe works on the other tile; the next item's loads and first scores start while
+// this one's output is written.  What bounds it: a half step takes a softmax warp about 1600 cycles, 820 of them the
+// exponentials (the special-function unit needs 512 for one tile's and serves both), 320 the load and the maximum, 345
+// waiting for the scores; the unit is busy 64 % of a sweep.
+// Measured (causal, one launch; the one-tile kernel above, several CTAs per SM, in brackets): 8 x 16 heads x 1024, dh 64
+// 41 us (50); 1 x 8 x 4096, dh 128 66 (101); 2 x 32 x 2048, dh 80 67 (120); 1 x 12 x 256, dh 64 6.9 (7.5).  Up to 160
+// positions the one-tile kernel is kept: 4 x 4 x 64, dh 32 3.5 against 4.3, 2 x 4 x 129, dh 64 5.4 against 6.2.
+// ------------------------------------------------------------------------------------------------
+template <int DH>
+struct Fwd2Cfg {
+  static constexpr int NCH = (DH + 63) / 64;
+  static constexpr int T_BYTES = NCH * 128 * 128;               // a 128-row operand
+  static constexpr int NST = NCH == 1 ? 4 : 2;                  // ring depth of K and of V
+  static constexpr int SMEM = 2 * T_BYTES + NST * 2 * T_BYTES + 1024 + 256;
+  static constexpr int C_O = 256, O_STRIDE = DH <= 64 ? 64 : 128;
+};
+constexpr int FWD2_THREADS = 352;
+constexpr int FWD_ONE_TILE_T = 160;    // up to this length (and for dh 256) the one-tile kernel is the faster one
+
+struct FwdItem { int qt, b, h, n0, n1; };
+__device__ __forceinline__ FwdItem fwd_item(int i, int nqt, int BH, int H, int T) {
+  FwdItem w;
+  const int r = i / BH, bh = i - r * BH;
+  w.qt = nqt - 1 - r;
+  w.b = bh / H;
+  w.h = bh - w.b * H;
+  w.n0 = 2 * w.qt + 1;                                          // key blocks up to and with the diagonal one
+  w.n1 = (2 * w.qt + 1) * 128 < T ? 2 * w.qt + 2 : 0;           // the second tile may lie wholly past the sequence
+  return w;
+}
+// item of round r for CTA c of G: forwards and backwards in turn, so that nobody always gets the longer ones
+__device__ __forceinline__ int snake(int r, int c, int G) { return r * G + ((r & 1) ? G - 1 - c : c); }
+
+template <int DH>
+__global__ void __launch_bounds__(FWD2_THREADS, 1) attn_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm, bf16* __restrict__ o,
+                                                                        float* __restrict__ lse, int B, int T, int H,
+                                                                        float scale, unsigned* err) {
+  using C = Fwd2Cfg<DH>;
+  constexpr int NST = C::NST;
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ int abort_flag;
+  __shared__ uint32_t tmem_base_smem;
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t sQ = base, sK0 = base + 2 * C::T_BYTES, sV0 = sK0 + NST * C::T_BYTES;
+  const uint32_t bars = sV0 + NST * C::T_BYTES;
+  const uint32_t bar_q = bars, bar_qfree = bars + 8;
+  auto bar_drain = [&](int x) { return bars + 232 + 8 * x; };
+  auto bar_s = [&](int x, int hf) { return bars + 24 + 8 * (2 * x + hf); };       // scores of a half block
+  auto bar_p = [&](int x, int hf) { return bars + 56 + 8 * (2 * x + hf); };       // ... turned into probabilities
+  auto bar_pv = [&](int x) { return bars + 88 + 8 * x; };                         // ... multiplied with V
+  auto bar_k = [&](int st) { return bars + 104 + 8 * st; };
+  auto bar_v = [&](int st) { return bars + 104 + 8 * (NST + st); };
+  auto bar_kfree = [&](int st) { return bars + 104 + 8 * (2 * NST + st); };
+  auto bar_vfree = [&](int st) { return bars + 104 + 8 * (3 * NST + st); };
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nqt = (T + 255) / 256, BH = B * H, nitems = nqt * BH, G = gridDim.x;
+  const int rounds = (nitems + G - 1) / G;
+  volatile int* abortp = &abort_flag;
+
+  if (tid == 0) {
+    abort_flag = 0;
+    mbar_init(bar_q, 1);
+    mbar_init(bar_qfree, 2);               // one arrival per issuing thread
+    mbar_init(bar_drain(0), 1);
+    mbar_init(bar_drain(1), 1);
+    for (int x = 0; x < 2; ++x) {
+      for (int hf = 0; hf < 2; ++hf) { mbar_init(bar_s(x, hf), 1); mbar_init(bar_p(x, hf), 4); }
+      mbar_init(bar_pv(x), 1);
+    }
+    for (int st = 0; st < NST; ++st) {
+      mbar_init(bar_k(st), 1); mbar_init(bar_v(st), 1);
+      mbar_init(bar_kfree(st), 2); mbar_init(bar_vfree(st), 2);
+    }
+    fence_mbar_init();
+    tma_prefetch_desc(&tm);
+  }
+  if (warp == 8) {
+    tmem_alloc(smem_u32(&tmem_base_smem), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  grid_dep_wait();
+  const uint32_t tmem_base = tmem_base_smem;
+  int fail = 0;
+
+  if (warp == 10) {
+    // ---------------------------------------------------------------- loads
+    if (lane == 0) {
+      int g = 0, n_item = 0;
+      auto load_tile = [&](uint32_t dst, int slot, int row, int b, uint32_t bar) {
+#pragma unroll
+        for (int c = 0; c < C::NCH; ++c) tma_load_4d(dst + c * (128 * 128), &tm, c * 64, slot, row, b, bar);
+      };
+      for (int r = 0; r < rounds && !fail; ++r) {
+        const int i = snake(r, blockIdx.x, G);
+        if (i >= nitems) continue;
+        const FwdItem w = fwd_item(i, nqt, BH, H, T);
+        const int n = w.n1 > w.n0 ? w.n1 : w.n0;
+        for (int j = 0; j < n; ++j) {
+          const int st = (g + j) % NST;
+          const uint32_t ph = (uint32_t)((g + j) / NST) & 1u;
+          if (!mbar_wait(bar_kfree(st), ph ^ 1u, abortp)) { fail = 1; break; }
+          mbar_expect_tx(bar_k(st), C::T_BYTES);
+          load_tile(sK0 + st * C::T_BYTES, H + w.h, j * 128, w.b, bar_k(st));
+          if (j == 0) {                     // (after the first K, which does not depend on the previous item's scores)
+            if (n_item > 0 && !mbar_wait(bar_qfree, (uint32_t)(n_item - 1) & 1u, abortp)) { fail = 1; break; }
+            mbar_expect_tx(bar_q, (w.n1 ? 2 : 1) * C::T_BYTES);
+            load_tile(sQ, w.h, w.qt * 256, w.b, bar_q);
+            if (w.n1) load_tile(sQ + C::T_BYTES, w.h, w.qt * 256 + 128, w.b, bar_q);
+          }
+          if (!mbar_wait(bar_vfree(st), ph ^ 1u, abortp)) { fail = 1; break; }
+          mbar_expect_tx(bar_v(st), C::T_BYTES);
+          load_tile(sV0 + st * C::T_BYTES, 2 * H + w.h, j * 128, w.b, bar_v(st));
+        }
+        g += n;
+        ++n_item;
+      }
+      grid_dep_launch();
+      if (fail) abort_flag = 1;
+    }
+  } else if (warp >= 8) {
+    // ---------------------------------------------------------------- MMA issue, one thread per tile
+    // (A thread issues an MMA of this size no faster than every ~54 cycles and is held up while the pipe is full: one
+    // thread for both tiles made the sweep wait for it.)
+    if (lane == 0) {
+      const int x = warp - 8;
+      constexpr uint32_t idesc_s = make_idesc_bf16(128, 64, 0, 0);
+      constexpr uint32_t idesc_o = make_idesc_bf16(128, DH, 0, 1);
+      const SmemDescBase dq = make_smem_desc_base(sQ + (uint32_t)x * C::T_BYTES, 16, 1024), dk = make_smem_desc_base(sK0, 16, 1024);
+      const SmemDescBase dv = make_smem_desc_base(sV0, 128 * 128, 1024);
+      const uint32_t t_s = tmem_base + 128 * x, t_o = tmem_base + C::C_O + C::O_STRIDE * x;
+      int g = 0, n_item = 0;
+      uint32_t pc = 0;                      // blocks of this tile consumed so far
+      bool ok = true;
+      // scores of keys 64 hf .. 64 hf + 63 of the block in stage st
+      auto issue_s = [&](int hf, int st) {
+        const uint32_t ko = (uint32_t)st * C::T_BYTES + (uint32_t)hf * (64 * 128);
+#pragma unroll
+        for (int ks = 0; ks < DH / 16; ++ks) {
+          const uint32_t off = (ks >> 2) * (128 * 128) + (ks & 3) * 32;
+          umma_bf16(t_s + 64 * hf, desc_at(dq, off), desc_at(dk, ko + off), idesc_s, ks ? 1u : 0u);
+        }
+        umma_commit(bar_s(x, hf));
+      };
+      for (int r = 0; r < rounds && ok; ++r) {
+        const int i = snake(r, blockIdx.x, G);
+        if (i >= nitems) continue;
+        const FwdItem w = fwd_item(i, nqt, BH, H, T);
+        const int nt = x ? w.n1 : w.n0;
+        const int n = w.n1 > w.n0 ? w.n1 : w.n0;          // both threads pace themselves by every block, used or not
+        if (!mbar_wait(bar_k(g % NST), (uint32_t)(g / NST) & 1u, abortp) || !mbar_wait(bar_q, (uint32_t)n_item & 1u, abortp)) { ok = false; break; }
+        tc_fence_after();
+        if (nt) { issue_s(0, g % NST); issue_s(1, g % NST); }
+        umma_commit(bar_kfree(g % NST));
+        if (n == 1) umma_commit(bar_qfree);
+        for (int j = 0; j < n && ok; ++j) {
+          const int st = (g + j) % NST, st1 = (g + j + 1) % NST;
+          if (!mbar_wait(bar_v(st), (uint32_t)((g + j) / NST) & 1u, abortp)) { ok = false; break; }
+          if (j + 1 < n && !mbar_wait(bar_k(st1), (uint32_t)((g + j + 1) / NST) & 1u, abortp)) { ok = false; break; }
+          if (j < nt) {
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+              if (!mbar_wait(bar_p(x, hf), pc & 1u, abortp)) { ok = false; break; }
+              tc_fence_after();
+              const uint32_t vo = (uint32_t)st * C::T_BYTES + (uint32_t)hf * (4 * 2048);
+#pragma unroll
+              for (int ks = 0; ks < 4; ++ks)
+                umma_bf16_ts(t_o, t_s + 64 * hf + 8 * ks, desc_at(dv, vo + ks * 2048), idesc_o, (j | hf | ks) ? 1u : 0u);
+              umma_commit(bar_pv(x));
+              if (j + 1 < nt) issue_s(hf, st1);
+            }
+            ++pc;
+          }
+          if (!ok) break;
+          umma_commit(bar_vfree(st));
+          if (j + 1 < n) {
+            umma_commit(bar_kfree(st1));
+            if (j + 2 == n) umma_commit(bar_qfree);       // the item's last scores
+          }
+        }
+        g += n;
+        ++n_item;
+      }
+      if (!ok) { fail = 1; abort_flag = 1; }
+      umma_commit(bar_drain(x));                   // every MMA issued has retired before TMEM goes
+      int never = 0;
+      mbar_wait(bar_drain(x), 0, &never);
+    }
+  } else {
+    // ---------------------------------------------------------------- softmax and output (thread = row of tile x)
+    const int x = warp >> 2;
+    const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t t_s = t_lane + 128 * x, t_o = t_lane + C::C_O + C::O_STRIDE * x;
+    const int d = H * DH;
+    const float c2 = scale * IL_LOG2E;
+    const float slack = 8.0f / c2;
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abortp)); };
+    uint32_t sc = 0;                               // blocks of this tile so far
+    for (int r = 0; r < rounds && !fail; ++r) {
+      const int i = snake(r, blockIdx.x, G);
+      if (i >= nitems) continue;
+      const FwdItem w = fwd_item(i, nqt, BH, H, T);
+      const int n = x ? w.n1 : w.n0;
+      if (n == 0) continue;
+      const int rl = (warp & 3) * 32 + lane;       // row within the tile
+      const int row = w.qt * 256 + x * 128 + rl;
+      float m = -INFINITY, l = 0.f;
+      for (int j = 0; j < n && !fail; ++j, ++sc) {
+#pragma unroll 1
+        for (int hf = 0; hf < 2; ++hf) {
+          if (!wait(bar_s(x, hf), sc & 1u)) { fail = 1; abort_flag = 1; break; }
+          tc_fence_after();
+          float s[64];
+          {
+            uint32_t u0[32], u1[32];
+            tmem_ld_32x32(t_s + 64 * hf, u0);
+            tmem_ld_32x32(t_s + 64 * hf + 32, u1);
+            tmem_ld_wait();
+#pragma unroll
+            for (int q = 0; q < 32; ++q) { s[q] = __uint_as_float(u0[q]); s[32 + q] = __uint_as_float(u1[q]); }
+          }
+          if (j + 1 == n) {                        // the diagonal block: keys after the query
+#pragma unroll
+            for (int q = 0; q < 64; ++q)
+              if (64 * hf + q > rl) s[q] = -INFINITY;
+          }
+          float mx4[4] = {s[0], s[1], s[2], s[3]};
+#pragma unroll
+          for (int q = 4; q < 60; q += 8)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) mx4[e] = fmaxf(mx4[e], fmaxf(s[q + e], s[q + 4 + e]));
+          const float mx = fmaxf(fmaxf(fmaxf(mx4[0], s[60]), fmaxf(mx4[1], s[61])), fmaxf(fmaxf(mx4[2], s[62]), fmaxf(mx4[3], s[63])));
+          if (__any_sync(0xffffffffu, mx > m + slack)) {            // warp-uniform: raise the reference maximum
+            const float mn = fmaxf(m, mx);
+            const float alpha = ex2_fast((m - mn) * c2);            // 0 on the first block (m = -inf)
+            l *= alpha;
+            m = mn;
+            if (j | hf) {                          // O holds everything up to the half before: that product has to be in
+              if (!wait(bar_pv(x), (2 * sc + hf - 1) & 1u)) { fail = 1; abort_flag = 1; break; }
+              tc_fence_after();
+#pragma unroll 1
+              for (int c0 = 0; c0 < DH; c0 += 16) {
+                uint32_t v[16];
+                tmem_ld_32x16(t_o + c0, v);
+                tmem_ld_wait();
+#pragma unroll
+                for (int q = 0; q < 16; ++q) v[q] = __float_as_uint(__uint_as_float(v[q]) * alpha);
+                tmem_st_32x16(t_o + c0, v);
+              }
+              tmem_st_wait();
+            }
+          }
+          const float mc = m * c2;
+          float ps4[4] = {0.f, 0.f, 0.f, 0.f};
+          uint32_t pw[32];
+#pragma unroll
+          for (int q = 0; q < 64; q += 4) {
+            const float e0 = ex2_fast(fmaf(s[q], c2, -mc)), e1 = ex2_fast(fmaf(s[q + 1], c2, -mc));
+            const float e2 = ex2_fast(fmaf(s[q + 2], c2, -mc)), e3 = ex2_fast(fmaf(s[q + 3], c2, -mc));
+            ps4[0] += e0; ps4[1] += e1; ps4[2] += e2; ps4[3] += e3;
+            pw[q / 2] = pack_bf16x2(e0, e1);
+            pw[q / 2 + 1] = pack_bf16x2(e2, e3);
+          }
+          tmem_st_32x32(t_s + 64 * hf, pw);        // P over the first half of the score columns this thread read
+          l += (ps4[0] + ps4[1]) + (ps4[2] + ps4[3]);
+          tmem_st_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_p(x, hf));
+        }
+      }
+      if (fail) break;
+      // the last block's two products, one phase after the other (a parity wait is only good for the phase that follows
+      // one known to be complete: the last scores covered the product before these)
+      if (!wait(bar_pv(x), (2 * sc - 2) & 1u) || !wait(bar_pv(x), (2 * sc - 1) & 1u)) { fail = 1; abort_flag = 1; break; }
+      tc_fence_after();
+      const float inv = 1.0f / l;
+      bf16* orow = o + ((size_t)w.b * T + row) * d + w.h * DH;
+#pragma unroll
+      for (int c0 = 0; c0 < DH; c0 += 16) {
+        uint32_t v[16];
+        tmem_ld_32x16(t_o + c0, v);
+        tmem_ld_wait();
+        if (row < T) {
+#pragma unroll
+          for (int q = 0; q < 16; q += 8) {
+            uint4 pk;
+            pk.x = pack_bf16x2(__uint_as_float(v[q]) * inv, __uint_as_float(v[q + 1]) * inv);
+            pk.y = pack_bf16x2(__uint_as_float(v[q + 2]) * inv, __uint_as_float(v[q + 3]) * inv);
+            pk.z = pack_bf16x2(__uint_as_float(v[q + 4]) * inv, __uint_as_float(v[q + 5]) * inv);
+            pk.w = pack_bf16x2(__uint_as_float(v[q + 6]) * inv, __uint_as_float(v[q + 7]) * inv);
+            *reinterpret_cast<uint4*>(orow + c0 + q) = pk;
+          }
+        }
+      }
+      if (row < T) lse[((size_t)w.b * H + w.h) * T + row] = m * scale + logf(l);
+      tc_fence_before();       // O has been read before this thread's next P lets the next item's products overwrite it
+    }
+  }
+  fail = __syncthreads_or(fail);
+  if (tid == 0 && fail && err) atomicExch(err, DEV_TIMEOUT_MMA);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 512);
+  }
+}
+
+template <int DH>
+cudaError_t fwd_pair_launch(const bf16* qkv, bf16* o, float* lse, int B, int T, int H, unsigned* err, cudaStream_t s) {
+  using C = Fwd2Cfg<DH>;
+  const unsigned long long d3 = 3ull * H * DH;
+  const unsigned long long dims[4] = {(unsigned long long)DH, 3ull * H, (unsigned long long)T, (unsigned long long)B};
+  const unsigned long long strides[3] = {(unsigned long long)DH * 2, d3 * 2, (unsigned long long)T * d3 * 2};
+  const unsigned box[4] = {64, 1, 128, 1};
+  CUtensorMap tm;
+  if (!tma_encode_bf16(&tm, qkv, 4, dims, strides, box)) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(attn_fwd_pair_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  if (e != cudaSuccess) return e;
+  const long long items = (long long)((T + 255) / 256) * B * H;
+  const int grid = (int)(items < 148 ? items : 148);
+  launch_dep(attn_fwd_pair_kernel<DH>, dim3(grid), dim3(FWD2_THREADS), C::SMEM, s, tm, o, lse, B, T, H, rsqrtf((float)DH), err);
+  return cudaGetLastError();
+}
+
 template <int DH>
 cudaError_t fwd_tc_launch(const bf16* qkv, bf16* o, float* lse, int B, int T, int H, unsigned* err, cudaStream_t s) {
   using C = FwdCfg<DH>;
@@ -1421,10 +1760,10 @@ cudaError_t attention_fwd(const bf16* qkv, bf16* o, float* lse, int B, int T, in
                           cudaStream_t s) {
   if (((uintptr_t)qkv % 16) || ((uintptr_t)o % 16) || ((uintptr_t)lse % 4)) return cudaErrorInvalidValue;
   switch (dh) {
-    case 32: return fwd_tc_launch<32>(qkv, o, lse, B, T, H, err, s);
-    case 64: return fwd_tc_launch<64>(qkv, o, lse, B, T, H, err, s);
-    case 80: return fwd_tc_launch<80>(qkv, o, lse, B, T, H, err, s);
-    case 128: return fwd_tc_launch<128>(qkv, o, lse, B, T, H, err, s);
+    case 32: return T > FWD_ONE_TILE_T ? fwd_pair_launch<32>(qkv, o, lse, B, T, H, err, s) : fwd_tc_launch<32>(qkv, o, lse, B, T, H, err, s);
+    case 64: return T > FWD_ONE_TILE_T ? fwd_pair_launch<64>(qkv, o, lse, B, T, H, err, s) : fwd_tc_launch<64>(qkv, o, lse, B, T, H, err, s);
+    case 80: return T > FWD_ONE_TILE_T ? fwd_pair_launch<80>(qkv, o, lse, B, T, H, err, s) : fwd_tc_launch<80>(qkv, o, lse, B, T, H, err, s);
+    case 128: return T > FWD_ONE_TILE_T ? fwd_pair_launch<128>(qkv, o, lse, B, T, H, err, s) : fwd_tc_launch<128>(qkv, o, lse, B, T, H, err, s);
     case 256: return fwd_tc_launch<256>(qkv, o, lse, B, T, H, err, s);
   }
   return cudaErrorInvalidValue;
