@@ -1775,6 +1775,7 @@ cudaError_t attention_bwd(const bf16* qkv, const bf16* o, const float* lse, cons
   if (((uintptr_t)qkv % 16) || ((uintptr_t)o % 16) || ((uintptr_t)dout % 16) || ((uintptr_t)dqkv % 16) ||
       ((uintptr_t)lse % 4) || ((uintptr_t)delta % 4))
     return cudaErrorInvalidValue;
+  if (T <= ATTN_BWD_SHORT_T) return attention_bwd_short(qkv, lse, dout, dqkv, NB, B, T, H, dh, err, s);
   if (dq_acc && (dh == 32 || dh == 64)) {        // one sweep, dQ summed over key tiles in the fp32 accumulator
     if ((uintptr_t)dq_acc % 16) return cudaErrorInvalidValue;
     return dh == 32 ? bwd_fused_launch<32>(qkv, o, lse, dout, dqkv, delta, dq_acc, NB, B, T, H, err, s)

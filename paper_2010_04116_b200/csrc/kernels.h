@@ -86,5 +86,10 @@ cudaError_t attention_fwd(const __nv_bfloat16* qkv, __nv_bfloat16* o, float* lse
 cudaError_t attention_bwd(const __nv_bfloat16* qkv, const __nv_bfloat16* o, const float* lse, const __nv_bfloat16* dout,
                           __nv_bfloat16* dqkv, float* delta, float* dq_acc, int NB, int B, int T, int H, int dh,
                           unsigned* err, cudaStream_t s);
+// ... of sequences of up to ATTN_BWD_SHORT_T positions, which attention_bwd sends here whatever dq_acc is: one kernel
+// without scratch whose sums all have a fixed order (attention_short.cu).
+constexpr int ATTN_BWD_SHORT_T = 128;
+cudaError_t attention_bwd_short(const __nv_bfloat16* qkv, const float* lse, const __nv_bfloat16* dout, __nv_bfloat16* dqkv,
+                                int NB, int B, int T, int H, int dh, unsigned* err, cudaStream_t s);
 
 }  // namespace il

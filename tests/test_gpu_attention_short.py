@@ -1,0 +1,44 @@
+"""Attention backward of short sequences (one 128 x 128 tile): edges of the 16-wide contraction steps and of the two 64-key halves,
+more items than resident CTAs, every head dimension."""
+import pytest
+
+torch = pytest.importorskip("torch")
+from paper_2010_04116_b200 import binding as il  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("dh", [32, 64, 80, 128, 256])
+@pytest.mark.parametrize("NB,B,T,H", [(1, 1, 2, 1), (2, 1, 15, 3), (2, 2, 16, 2), (4, 2, 17, 2), (3, 3, 63, 4), (2, 1, 64, 2), (2, 2, 65, 3),
+                                      (1, 1, 113, 2), (2, 1, 127, 2), (160, 80, 128, 4), (301, 301, 40, 1)])
+def test_short_backward_matches_fp64(NB, B, T, H, dh):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(NB * T + dh)
+    d = H * dh
+    qkv = torch.randn(B * T, 3 * d, device=DEV, generator=g).to(torch.bfloat16)
+    dout = torch.randn(NB * T, d, device=DEV, generator=g).to(torch.bfloat16)
+    q, k, v = (x.permute(0, 2, 1, 3).double() for x in qkv.view(B, T, 3, H, dh).unbind(2))
+    s = (q @ k.transpose(-1, -2)) / dh ** 0.5
+    s = s.masked_fill(torch.ones(T, T, device=DEV, dtype=torch.bool).triu(1), float("-inf"))
+    lse = torch.logsumexp(s, -1)
+    idx = torch.arange(NB, device=DEV) % B
+    p = torch.softmax(s, -1)[idx]
+    do = dout.view(NB, T, H, dh).permute(0, 2, 1, 3).double()
+    dp = do @ v[idx].transpose(-1, -2)
+    ds = p * (dp - (p * dp).sum(-1, keepdim=True)) / dh ** 0.5
+    ref = torch.stack([ds @ k[idx], ds.transpose(-1, -2) @ q[idx], p.transpose(-1, -2) @ do])        # [3, NB, H, T, dh]
+    ref = ref.permute(1, 3, 0, 2, 4).reshape(NB * T, 3 * d)
+    got = torch.full((NB * T, 3 * d), 7.0, device=DEV, dtype=torch.bfloat16)
+    o = torch.zeros(B * T, d, device=DEV, dtype=torch.bfloat16)
+    delta = torch.zeros(NB * H * T, device=DEV)
+    il.op_attention_bwd(qkv, o, lse.float(), dout, got, delta, NB, B, T, H, dh)
+    torch.cuda.synchronize()
+    for i in range(3):
+        a, b = got[:, i * d:(i + 1) * d].double(), ref[:, i * d:(i + 1) * d]
+        # P or dS and the result are rounded to bf16, 2^-9 / sqrt(3) each in the mean: together 0.82 * 2^-9
+        assert float((a - b).norm() / b.norm()) < 2.0 ** -8, "qkv"[i]
+    again = torch.full((NB * T, 3 * d), -3.0, device=DEV, dtype=torch.bfloat16)
+    il.op_attention_bwd(qkv, o, lse.float(), dout, again, delta, NB, B, T, H, dh)
+    torch.cuda.synchronize()
+    assert torch.equal(got, again)                # every sum has a fixed order
