@@ -299,7 +299,7 @@ struct Fwd2Cfg {
   static constexpr int NCH = (DH + 63) / 64;
   static constexpr int T_BYTES = NCH * 128 * 128;               // a 128-row operand
   static constexpr int NST = NCH == 1 ? 4 : 2;                  // ring depth of K and of V
-  static constexpr int SMEM = 2 * T_BYTES + NST * 2 * T_BYTES + 1024 + 256;
+  static constexpr int SMEM = 2 * T_BYTES + NST * 2 * T_BYTES + 1024 + 512;
   static constexpr int C_O = 256, O_STRIDE = DH <= 64 ? 64 : 128;
 };
 constexpr int FWD2_THREADS = 352;
@@ -332,14 +332,17 @@ __global__ void __launch_bounds__(FWD2_THREADS, 1) attn_fwd_pair_kernel(const __
   const uint32_t sQ = base, sK0 = base + 2 * C::T_BYTES, sV0 = sK0 + NST * C::T_BYTES;
   const uint32_t bars = sV0 + NST * C::T_BYTES;
   const uint32_t bar_q = bars, bar_qfree = bars + 8;
-  auto bar_drain = [&](int x) { return bars + 232 + 8 * x; };
+  auto bar_drain = [&](int x) { return bars + 16 * NST * 2 + 120 + 8 * x; };
   auto bar_s = [&](int x, int hf) { return bars + 24 + 8 * (2 * x + hf); };       // scores of a half block
   auto bar_p = [&](int x, int hf) { return bars + 56 + 8 * (2 * x + hf); };       // ... turned into probabilities
-  auto bar_pv = [&](int x) { return bars + 88 + 8 * x; };                         // ... multiplied with V
-  auto bar_k = [&](int st) { return bars + 104 + 8 * st; };
-  auto bar_v = [&](int st) { return bars + 104 + 8 * (NST + st); };
-  auto bar_kfree = [&](int st) { return bars + 104 + 8 * (2 * NST + st); };
-  auto bar_vfree = [&](int st) { return bars + 104 + 8 * (3 * NST + st); };
+  // ... multiplied with V.  One barrier per half: whoever waits for a phase by its parity must know that the phase before it is
+  // over and that the one after it cannot be, and a softmax warp held up between its arrival and its wait can find both
+  // halves' products done.
+  auto bar_pv = [&](int x, int hf) { return bars + 88 + 8 * (2 * x + hf); };
+  auto bar_k = [&](int st) { return bars + 120 + 8 * st; };
+  auto bar_v = [&](int st) { return bars + 120 + 8 * (NST + st); };
+  auto bar_kfree = [&](int st) { return bars + 120 + 8 * (2 * NST + st); };
+  auto bar_vfree = [&](int st) { return bars + 120 + 8 * (3 * NST + st); };
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nqt = (T + 255) / 256, BH = B * H, nitems = nqt * BH, G = gridDim.x;
@@ -353,8 +356,7 @@ __global__ void __launch_bounds__(FWD2_THREADS, 1) attn_fwd_pair_kernel(const __
     mbar_init(bar_drain(0), 1);
     mbar_init(bar_drain(1), 1);
     for (int x = 0; x < 2; ++x) {
-      for (int hf = 0; hf < 2; ++hf) { mbar_init(bar_s(x, hf), 1); mbar_init(bar_p(x, hf), 4); }
-      mbar_init(bar_pv(x), 1);
+      for (int hf = 0; hf < 2; ++hf) { mbar_init(bar_s(x, hf), 1); mbar_init(bar_p(x, hf), 4); mbar_init(bar_pv(x, hf), 1); }
     }
     for (int st = 0; st < NST; ++st) {
       mbar_init(bar_k(st), 1); mbar_init(bar_v(st), 1);
@@ -457,7 +459,7 @@ __global__ void __launch_bounds__(FWD2_THREADS, 1) attn_fwd_pair_kernel(const __
 #pragma unroll
               for (int ks = 0; ks < 4; ++ks)
                 umma_bf16_ts(t_o, t_s + 64 * hf + 8 * ks, desc_at(dv, vo + ks * 2048), idesc_o, (j | hf | ks) ? 1u : 0u);
-              umma_commit(bar_pv(x));
+              umma_commit(bar_pv(x, hf));
               if (j + 1 < nt) issue_s(hf, st1);
             }
             ++pc;
@@ -527,7 +529,7 @@ __global__ void __launch_bounds__(FWD2_THREADS, 1) attn_fwd_pair_kernel(const __
             l *= alpha;
             m = mn;
             if (j | hf) {                          // O holds everything up to the half before: that product has to be in
-              if (!wait(bar_pv(x), (2 * sc + hf - 1) & 1u)) { fail = 1; abort_flag = 1; break; }
+              if (!wait(bar_pv(x, hf ^ 1), (hf ? sc : sc - 1) & 1u)) { fail = 1; abort_flag = 1; break; }
               tc_fence_after();
 #pragma unroll 1
               for (int c0 = 0; c0 < DH; c0 += 16) {
@@ -561,9 +563,8 @@ __global__ void __launch_bounds__(FWD2_THREADS, 1) attn_fwd_pair_kernel(const __
         }
       }
       if (fail) break;
-      // the last block's two products, one phase after the other (a parity wait is only good for the phase that follows
-      // one known to be complete: the last scores covered the product before these)
-      if (!wait(bar_pv(x), (2 * sc - 2) & 1u) || !wait(bar_pv(x), (2 * sc - 1) & 1u)) { fail = 1; abort_flag = 1; break; }
+      // the last block's two products (the block before it is done: its products precede the last scores in the pipe)
+      if (!wait(bar_pv(x, 0), (sc - 1) & 1u) || !wait(bar_pv(x, 1), (sc - 1) & 1u)) { fail = 1; abort_flag = 1; break; }
       tc_fence_after();
       const float inv = 1.0f / l;
       bf16* orow = o + ((size_t)w.b * T + row) * d + w.h * DH;

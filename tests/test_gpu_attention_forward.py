@@ -33,3 +33,27 @@ def test_forward_matches_fp64(B, T, H, dh):
     rows = (o.double() - ref).norm(dim=1) / ref.norm(dim=1)
     assert float(rows.max()) < 2.0 ** -6                      # no single row is off by more than a few roundings
     assert float((lse.double() - torch.logsumexp(s, -1)).abs().max()) < 2e-4      # ex2.approx and fp32 sums at |lse| up to ~100
+
+
+def test_forward_beside_another_streams_traffic():
+    """Many launches while another stream keeps the memory and the SMs busy: no warp may miss a barrier phase however late it
+    comes to wait for it (a CTA whose wait runs out leaves its later items unwritten)."""
+    B, T, H, dh = 5, 501, 16, 32                     # two items for some of the CTAs
+    d = H * dh
+    qkv = torch.randn(B * T, 3 * d, device=DEV).to(torch.bfloat16)
+    big = torch.zeros(64 << 20, device=DEV)
+    outs = [torch.zeros(B * T, d, device=DEV, dtype=torch.bfloat16) for _ in range(2)]
+    lse = torch.zeros(B, H, T, device=DEV)
+    il.op_attention_fwd(qkv, outs[0], lse, B, T, H, dh)
+    torch.cuda.synchronize()
+    ref = outs[0].clone()
+    side = torch.cuda.Stream()
+    for _ in range(40):
+        with torch.cuda.stream(side):
+            for _ in range(4):
+                big.add_(1.0)
+        for i in range(50):
+            outs[1].fill_(7.0)
+            il.op_attention_fwd(qkv, outs[1], lse, B, T, H, dh, stream=torch.cuda.current_stream().cuda_stream)
+        assert torch.equal(outs[1], ref)
+    torch.cuda.synchronize()
