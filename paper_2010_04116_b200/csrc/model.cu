@@ -137,7 +137,8 @@ struct il_model {
   std::vector<int*> tokens, targets;  // per component: the batch on that component's device (shared on one device)
   std::vector<float*> losses;         // per component: device [K] array holding losses[k] at index k
   // Error words, per component (shared on one device): word 0 = DEV_* code of the first failure, words 1..K =
-  // number of AdamW updates component k-1 applied since the last il_sync (an update is skipped while word 0 is set).
+  // number of AdamW updates component k-1 applied since the last il_sync (an update is skipped while word 0 is set), words
+  // K+1..2K = the same of its head's vocabulary matrix.
   std::vector<unsigned*> err_word;
   // pipeline placement: receive buffers owned by the component's device
   std::vector<float*> a_in;           // a_{k}: input of component k (k >= 1), copied from component k-1's output
@@ -755,8 +756,8 @@ extern "C" il_status il_create(int K, int Lc, int d, int H, int F, int V, int n,
     IL_TRY(dev_alloc_t(m, &m->tokens[k], N));
     IL_TRY(dev_alloc_t(m, &m->targets[k], N));
     IL_TRY(dev_alloc_t(m, &m->losses[k], (size_t)K));
-    IL_TRY(dev_alloc_t(m, &m->err_word[k], (size_t)(1 + K)));
-    IL_CUDA(m, cudaMemsetAsync(m->err_word[k], 0, 4 * (1 + K), m->streams[k]));
+    IL_TRY(dev_alloc_t(m, &m->err_word[k], (size_t)(1 + 2 * K)));
+    IL_CUDA(m, cudaMemsetAsync(m->err_word[k], 0, 4 * (1 + 2 * K), m->streams[k]));
     IL_CUDA(m, cudaMemsetAsync(m->losses[k], 0, K * 4, m->streams[k]));
   }
   IL_CUDA(m, cudaSetDevice(m->dev[0]));
@@ -1540,10 +1541,15 @@ extern "C" il_status il_adamw_step(il_model* m, float lr, float beta1, float bet
     cudaStream_t hs = aside ? m->side[k] : m->streams[k];
     if (aside) IL_CUDA(m, cudaStreamWaitEvent(hs, m->ev_head[k], 0));
     IL_K(m, adamw(m->P[k] + hw0, m->M1[k] + hw0, m->M2[k] + hw0, m->G[k] + hw0, m->Pb[k] + hw0, hw1 - hw0, hw1 - hw0, lr, beta1, beta2,
-                  eps, wd, (float)bc1, (float)bc2, m->err_word[k], nullptr, 0, 0, hs));
-    if (aside) IL_CUDA(m, cudaEventRecord(m->ev_side[k], hs));
+                  eps, wd, (float)bc1, (float)bc2, m->err_word[k], m->err_word[k] + 1 + m->K + k, (unsigned)m->adamw_issued, 0, 0, aside, hs));
+    // the rest of the component follows there too while lower components' backward passes go on
+    const bool later = aside && k > 0;
+    cudaStream_t ts = later ? hs : m->streams[k];
+    if (later) IL_CUDA(m, cudaStreamWaitEvent(ts, m->ev_bwd[k], 0));
+    else if (aside) IL_CUDA(m, cudaEventRecord(m->ev_side[k], hs));
     IL_K(m, adamw(m->P[k] + b, m->M1[k] + b, m->M2[k] + b, m->G[k] + b, m->Pb[k] + b, e - b, me - b, lr, beta1, beta2, eps, wd,
-                  (float)bc1, (float)bc2, m->err_word[k], m->err_word[k] + 1 + k, hw0 - b, hw1 - b, m->streams[k]));
+                  (float)bc1, (float)bc2, m->err_word[k], m->err_word[k] + 1 + k, (unsigned)m->adamw_issued, hw0 - b, hw1 - b, later, ts));
+    if (later) IL_CUDA(m, cudaEventRecord(m->ev_side[k], hs));
     if (aside) IL_CUDA(m, cudaStreamWaitEvent(m->streams[k], m->ev_side[k], 0));   // stream k's tail covers the side stream
   }
   m->batch_set = false;   // a new batch is required for the next step
@@ -1572,7 +1578,7 @@ extern "C" il_status il_sync(il_model* m) {
       applied_min = std::min(applied_min, (int)words[1 + j]);
       applied_max = std::max(applied_max, (int)words[1 + j]);
     }
-    IL_CUDA(m, cudaMemsetAsync(m->err_word[k], 0, 4 * (size_t)(1 + m->K), m->streams[k]));
+    IL_CUDA(m, cudaMemsetAsync(m->err_word[k], 0, 4 * (size_t)(1 + 2 * m->K), m->streams[k]));
     IL_CUDA(m, cudaStreamSynchronize(m->streams[k]));
   }
   const int issued = m->adamw_issued;
