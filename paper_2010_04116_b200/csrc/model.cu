@@ -946,12 +946,7 @@ extern "C" il_status il_set_batch(il_model* m, const int* tokens, const int* tar
     IL_CUDA(m, cudaMemcpyAsync(m->targets[k], targets, bytes, kind, m->streams[k]));
   }
   IL_CUDA(m, cudaSetDevice(m->dev[0]));
-  // (token, position) keys in sorted order for the embedding backward: made on component 0's side stream beside the
-  // forward pass (44 us for 8192 positions, which would otherwise precede every step's first kernel)
   IL_CUDA(m, cudaEventRecord(m->ev_batch, s0));
-  IL_CUDA(m, cudaStreamWaitEvent(m->side[0], m->ev_batch, 0));
-  IL_K(m, embed_sort(m->tokens[0], m->sort_keys[0], B * T, m->V, m->side[0]));
-  IL_CUDA(m, cudaEventRecord(m->ev_sort, m->side[0]));
   if (m->tokens[1 % m->K] == m->tokens[0]) {     // shared buffers: the other streams start after the copies
     for (int k = 1; k < m->K; ++k) IL_CUDA(m, cudaStreamWaitEvent(m->streams[k], m->ev_batch, 0));
   }
@@ -1228,7 +1223,7 @@ il_status layers_backward(il_model* m, int k, int s, size_t base, int count, con
     IL_TRY(br.join(1));                          // dbig (and, since the last block's mark came before, dqkv) is replaced
     IL_K(m, attention_bwd(A.qkv, A.attn_o, A.lse, c.dattn, c.dqkv, c.delta, dq_acc, s * m->B, m->B, m->T, m->H, m->dh,
                           m->err_word[k], st));
-    m->launches += 2;
+    if (m->T > ATTN_BWD_SHORT_T) m->launches += 2;
     IL_TRY(br.fork());
     IL_K(m, colsum_bf16(c.dqkv, 3 * d, m->G[k] + o.bqkv, N, 3 * d, br.st));
     IL_TRY(wgrad(m, k, 3 * d, d, N, c.dqkv, 3 * d, A.ln1, d, m->G[k] + o.wqkv, acc, br.st));
@@ -1264,6 +1259,14 @@ il_status head_backward(il_model* m, int k, bool acc, float scale) {
   // the GPU idle on small batches, is planned as one of (at least) two that run side by side
   const int beside = m->placement == IL_PLACE_SINGLE && m->K > 1 ? 2 : 1;
   BackwardBranch br(m, k, N, d);
+  if (!acc) {   // vectors are summed into atomically; embedding rows no token selects must read zero
+    IL_TRY(br.fork());
+    IL_CUDA(m, cudaMemsetAsync(m->G[k] + m->comp_mat_end[k], 0, (m->comp_end[k] - m->comp_mat_end[k]) * 4, br.st));
+    if (k == 0) {
+      IL_CUDA(m, cudaMemsetAsync(m->G[k] + m->off_wte, 0, (size_t)V * d * 4, br.st));
+      IL_CUDA(m, cudaMemsetAsync(m->G[k] + m->off_wpe, 0, (size_t)m->max_seq * d * 4, br.st));
+    }
+  }
   if (m->head_mode == IL_HEAD_STORED) {
     IL_K(m, head_backward_prepare(h.z, m->ldz, h.lse, m->targets[k], h.u, h.us, h.rs, N, d, scale, m->err_word[k], st));
     {  // dU = diag(s) (E' W).  Not split over the contraction: atomically added partial sums would make dU, and
@@ -1309,26 +1312,36 @@ il_status head_backward(il_model* m, int k, bool acc, float scale) {
     }
   }
   const float* hx = head_input(m, k);
-  IL_TRY(br.fork());
-  IL_K(m, layernorm_bwd_params(h.du, 1, hx, h.mean, h.rstd, m->G[k] + o.lng, m->G[k] + o.lnb, N, d, br.st));
-  IL_TRY(br.mark(2));
+  IL_TRY(br.mark(2));              // (the vectors' zeroes and dW)
+  IL_TRY(br.join(2));
+  IL_K(m, layernorm_bwd_params(h.du, 1, hx, h.mean, h.rstd, m->G[k] + o.lng, m->G[k] + o.lnb, N, d, st));
   if (m->Lh == 0) {
     IL_K(m, layernorm_bwd_rows(h.du, 1, hx, h.mean, h.rstd, m->P[k] + o.lng, nullptr, h.ghead, nullptr, N, N, d, st));
-    IL_TRY(br.join(2));
     return IL_OK;
   }
   CompScratch& c = m->cs[k];
   IL_K(m, layernorm_bwd_rows(h.du, 1, hx, h.mean, h.rstd, m->P[k] + o.lng, nullptr, c.dx, c.dxb, N, N, d, st));
-  IL_TRY(br.join(2));
   IL_TRY(layers_backward(m, k, 1, (size_t)m->K * m->Lc + (size_t)k * m->Lh, m->Lh, m->a[k + 1], acc));
   IL_CUDA(m, cudaMemcpyAsync(h.ghead, c.dx, (size_t)N * d * sizeof(float), cudaMemcpyDeviceToDevice, st));
   return IL_OK;
 }
 
-il_status component_backward(il_model* m, int k, int s, bool acc) {
-  const int key[6] = {m->B, m->T, s, acc ? 1 : 0, 0, 0};
+// Backward of component k for s stacked gradient streams, which `gather` puts in place (kernels on stream k that depend on
+// nothing but the rule and the window), down to the embedding's gradients below component 0.
+template <class G>
+il_status component_backward(il_model* m, int k, int s, bool acc, G&& gather) {
+  cudaStream_t st = m->streams[k];
+  if (k == 0) IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_sort, 0));
+  const int key[6] = {m->B, m->T, s, acc ? 1 : 0, m->n, m->rule};
   return run_segment(m, SEG_COMPONENT_BACKWARD, k, key, [&]() -> il_status {
-    return layers_backward(m, k, s, (size_t)k * m->Lc, m->Lc, comp_input(m, k), acc);
+    IL_TRY(gather());
+    IL_TRY(layers_backward(m, k, s, (size_t)k * m->Lc, m->Lc, comp_input(m, k), acc));
+    if (k == 0) {
+      IL_K(m, embed_bwd(m->tokens[k], m->sort_keys[0], m->cs[0].dx, m->G[k] + m->off_wte, m->G[k] + m->off_wpe, m->ntok, m->T, m->d,
+                        m->V, acc ? 1 : 0, st));
+      m->launches++;
+    }
+    return IL_OK;
   });
 }
 
@@ -1373,14 +1386,6 @@ extern "C" il_status il_backward_nwise(il_model* m) {
   for (int k = 0; k < K; ++k) {
     cudaStream_t st = m->streams[k];
     IL_CUDA(m, cudaSetDevice(m->dev[k]));
-    if (!acc) {   // vectors are summed into atomically; embedding rows no token selects must read zero
-      IL_CUDA(m, cudaMemsetAsync(m->G[k] + m->comp_mat_end[k], 0, (m->comp_end[k] - m->comp_mat_end[k]) * 4, st));
-      if (k == 0) {
-        const size_t emb = (size_t)m->V * d;
-        IL_CUDA(m, cudaMemsetAsync(m->G[k] + m->off_wte, 0, emb * 4, st));
-        IL_CUDA(m, cudaMemsetAsync(m->G[k] + m->off_wpe, 0, (size_t)m->max_seq * d * 4, st));
-      }
-    }
     {
       Range r2("head backward %d", k);
       const int key[6] = {m->B, m->T, m->head_mode, acc ? 1 : 0, m->micro, 0};
@@ -1388,6 +1393,12 @@ extern "C" il_status il_backward_nwise(il_model* m) {
     }
     IL_CUDA(m, cudaEventRecord(m->ev_head[k], st));      // head k's parameter gradients are final from here on
   }
+  // (token, position) keys in sorted order for the embedding backward: made on component 0's side stream beside all that comes
+  // before it (44 us for 8192 positions; a forward pass without a backward does not need them)
+  IL_CUDA(m, cudaSetDevice(m->dev[0]));
+  IL_CUDA(m, cudaStreamWaitEvent(m->side[0], m->ev_batch, 0));
+  IL_K(m, embed_sort(m->tokens[0], m->sort_keys[0], N, m->V, m->side[0]));
+  IL_CUDA(m, cudaEventRecord(m->ev_sort, m->side[0]));
   if (m->rule == IL_RULE_SUM) {
     // components from the top down; component k needs the pass-down of component k+1 when any stream crosses
     std::vector<int> above;   // termination levels of the streams of component k+1
@@ -1397,6 +1408,7 @@ extern "C" il_status il_backward_nwise(il_model* m) {
       fetched.assign((size_t)m->s_cap + 1, 0);
       const std::vector<int> terms = terms_of(k, K, n);
       const int s = (int)terms.size();
+      std::vector<const float*> pass(s);
       bool needs_above = false;
       for (int j = 0; j < s; ++j) {
         int src = -1;
@@ -1406,18 +1418,16 @@ extern "C" il_status il_backward_nwise(il_model* m) {
           IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_bwd[k + 1], 0));
           needs_above = true;
         }
-        const float* passed = src >= 0 ? from_above(k, src, terms[j]) : nullptr;
+        pass[j] = src >= 0 ? from_above(k, src, terms[j]) : nullptr;
         if (fetch_err != cudaSuccess) return fail(m, IL_ERR_CUDA, "cudaMemcpyPeerAsync: %s", cudaGetErrorString(fetch_err));
-        IL_K(m, add_convert(m->hs[k].ghead, passed, m->cs[k].dx + (size_t)j * slice, m->cs[k].dxb + (size_t)j * slice, slice, st));
       }
       {
         Range r2("component backward %d", k);
-        IL_TRY(component_backward(m, k, s, acc));
-      }
-      if (k == 0) {
-        IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_sort, 0));
-        IL_K(m, embed_bwd(m->tokens[k], m->sort_keys[0], m->cs[0].dx, m->G[k] + m->off_wte, m->G[k] + m->off_wpe, N, m->T, d, m->V, acc ? 1 : 0, st));
-        m->launches++;
+        IL_TRY(component_backward(m, k, s, acc, [&]() -> il_status {
+          for (int j = 0; j < s; ++j)
+            IL_K(m, add_convert(m->hs[k].ghead, pass[j], m->cs[k].dx + (size_t)j * slice, m->cs[k].dxb + (size_t)j * slice, slice, st));
+          return IL_OK;
+        }));
       }
       IL_CUDA(m, cudaEventRecord(m->ev_bwd[k], st));
       above = terms;
@@ -1443,10 +1453,10 @@ extern "C" il_status il_backward_nwise(il_model* m) {
       if (hi > k) IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_bwd[k + 1], 0));
       // slot 0: the weighted combination
       int single = -1;                  // the head slot 0 equals exactly, if any
+      const float* xs[8];
+      float ws[8];
+      int cnt = 0;
       {
-        const float* xs[8];
-        float ws[8];
-        int cnt = 0;
         for (int h = k; h <= hi; ++h) {
           const float wgt = rule_weight(m->rule, k, h, n, K);
           if (wgt == 0.0f) continue;
@@ -1455,13 +1465,10 @@ extern "C" il_status il_backward_nwise(il_model* m) {
           single = (cnt == 0 && wgt == 1.0f) ? h : -1;
           ws[cnt++] = wgt;
         }
-        for (int c0 = 0; c0 < cnt; c0 += 4) {
-          const int c = cnt - c0 < 4 ? cnt - c0 : 4;
-          IL_K(m, lincomb_convert(xs + c0, ws + c0, c, c0 > 0, m->cs[k].dx, c0 + 4 >= cnt ? m->cs[k].dxb : nullptr, slice, st));
-        }
       }
       // slots 1..: heads that continue below this component
       std::vector<int> mine, mine_slots;
+      std::vector<const float*> relay{nullptr};        // source of each slot from 1 on
       int used = 1;
       if (k > 0)
         for (int h = k; h <= hi; ++h)
@@ -1470,18 +1477,21 @@ extern "C" il_status il_backward_nwise(il_model* m) {
             if (h == single) { mine_slots.push_back(0); continue; }
             const float* src = grad_of(h);
             if (!src) return fail(m, IL_ERR_STATE, "internal: gradient stream of head %d missing at component %d", h, k);
-            IL_K(m, add_convert(src, nullptr, m->cs[k].dx + (size_t)used * slice, m->cs[k].dxb + (size_t)used * slice, slice, st));
+            relay.push_back(src);
             mine_slots.push_back(used++);
           }
       if (fetch_err != cudaSuccess) return fail(m, IL_ERR_CUDA, "cudaMemcpyPeerAsync: %s", cudaGetErrorString(fetch_err));
       {
         Range r2("component backward %d", k);
-        IL_TRY(component_backward(m, k, used, acc));
-      }
-      if (k == 0) {
-        IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_sort, 0));
-        IL_K(m, embed_bwd(m->tokens[k], m->sort_keys[0], m->cs[0].dx, m->G[k] + m->off_wte, m->G[k] + m->off_wpe, N, m->T, d, m->V, acc ? 1 : 0, st));
-        m->launches++;
+        IL_TRY(component_backward(m, k, used, acc, [&]() -> il_status {
+          for (int c0 = 0; c0 < cnt; c0 += 4) {
+            const int c = cnt - c0 < 4 ? cnt - c0 : 4;
+            IL_K(m, lincomb_convert(xs + c0, ws + c0, c, c0 > 0, m->cs[k].dx, c0 + 4 >= cnt ? m->cs[k].dxb : nullptr, slice, st));
+          }
+          for (int j = 1; j < used; ++j)
+            IL_K(m, add_convert(relay[j], nullptr, m->cs[k].dx + (size_t)j * slice, m->cs[k].dxb + (size_t)j * slice, slice, st));
+          return IL_OK;
+        }));
       }
       IL_CUDA(m, cudaEventRecord(m->ev_bwd[k], st));
       above_heads = mine;
