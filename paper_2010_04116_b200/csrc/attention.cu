@@ -635,29 +635,27 @@ cudaError_t fwd_tc_launch(const bf16* qkv, bf16* o, float* lse, int B, int T, in
 
 
 // ------------------------------------------------------------------------------------------------
-// Backward.  Same structure as the forward: a CTA owns 128 rows (keys for dK/dV, queries for dQ), the other
-// index is swept in blocks of 64; two threads share a row (32 columns of each block each: the backward has
+// Backward at head dimension 256 (the smaller ones: attention_sweep.cu).  Same structure as the forward: a CTA owns 128 rows
+// (keys for dK/dV, queries for dQ), the other index is swept in blocks of 64; two threads share a row (32 columns of each block each: the backward has
 // no row-wise reduction, so they never need to talk), all products run on tcgen05 and
 // — because the backward has no running maximum — every gradient accumulates in TMEM across the sweep.
 // Probabilities are recomputed from the saved log-sum-exp; delta_i = sum_c dO_ic O_ic.
 // P^T and dS^T (dS for dQ) never touch shared memory: a thread rounds its 32 values to bf16, packs them in
 // pairs and stores the 16 words back into the first half of the TMEM columns it has just read, from where
-// the next MMA takes them as its A operand.  The tiles of the swept index come through a 4-deep TMA ring.
+// the next MMA takes them as its A operand.  One 64 KB stage of swept tiles is all that fits beside the row operands, so a
+// step's scores are issued at its own top; dV and dK do not fit the 512 TMEM columns together and run as two launches.
 // ------------------------------------------------------------------------------------------------
 
 template <int DH>
 struct BwdCfg {
   static constexpr int NCH = (DH + 63) / 64;
-  static constexpr int NST = (DH > 128) ? 1 : 4;        // ring depth of the swept tiles (one 64 KB stage is all that fits at dh 256)
-  static constexpr bool AHEAD = NST > 1;                // the next step's scores are issued one step ahead (needs a second stage)
   static constexpr int ROW_BYTES = NCH * TQ * 128;      // a 128-row operand (all chunks)
   static constexpr int BLK_BYTES = NCH * TK * 128;      // a 64-row operand
-  // dK/dV: K, V resident; ring of (Q, dO); lse/delta vectors.  TMEM: S^T, dP^T, dV, dK.
-  static constexpr int SMEM_KV = 2 * ROW_BYTES + NST * 2 * BLK_BYTES + 1024 + 2 * 2 * 64 * 4 + 128;
-  static constexpr int TCOLS_KV = (128 + 2 * DH <= 256) ? 256 : 512;   // dh 256: one accumulator per launch (PART)
-  // dQ: Q, dO resident; ring of (K, V).  TMEM: S, dP, dQ.
-  static constexpr int SMEM_Q = 2 * ROW_BYTES + NST * 2 * BLK_BYTES + 1024 + 128;
-  static constexpr int TCOLS_Q = (128 + DH <= 256) ? 256 : 512;
+  // dK/dV: K, V resident; one stage of (Q, dO); lse/delta vectors.  TMEM: S^T, dP^T, dV or dK.
+  static constexpr int SMEM_KV = 2 * ROW_BYTES + 2 * BLK_BYTES + 1024 + 2 * 2 * 64 * 4 + 128;
+  // dQ: Q, dO resident; one stage of (K, V).  TMEM: S, dP, dQ.
+  static constexpr int SMEM_Q = 2 * ROW_BYTES + 2 * BLK_BYTES + 1024 + 128;
+  static constexpr int TCOLS = 512;
 };
 
 // 32 fp32 values -> 16 words of bf16 pairs (even index in the low half)
@@ -669,8 +667,7 @@ __device__ __forceinline__ void pack_row32(const float (&v)[32], uint32_t (&w)[1
 // their first 16 columns) of the A operand of K-step ks (16 elements = 8 columns)
 __device__ __forceinline__ constexpr uint32_t packed_col(int ks) { return (uint32_t)((ks >> 1) * 32 + (ks & 1) * 8); }
 
-// PART: 0 = dV and dK in one launch; 1 = dV only; 2 = dK only (head dimensions whose two accumulators do not fit
-// the 512 TMEM columns together run as two launches, each recomputing the scores).
+// PART: 1 = dV, 2 = dK (each recomputing the scores).
 template <int DH, int PART>
 __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmRow,   // qkv, 128-row box
                                                               const __grid_constant__ CUtensorMap tmBlk,   // qkv, 64-row box
@@ -679,14 +676,13 @@ __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_const
                                                               bf16* __restrict__ dqkv, int B, int T, int H, float scale,
                                                               unsigned* err) {
   using C = BwdCfg<DH>;
-  constexpr int NST = C::NST;
   extern __shared__ uint8_t smem_raw[];
   __shared__ int abort_flag;
   __shared__ uint32_t tmem_base_smem;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sK = base, sV = sK + C::ROW_BYTES;
-  const uint32_t sQ0 = sV + C::ROW_BYTES, sdO0 = sQ0 + NST * C::BLK_BYTES;
-  const uint32_t vecs = sdO0 + NST * C::BLK_BYTES;               // lse2[2][64], delta[2][64]
+  const uint32_t sQ0 = sV + C::ROW_BYTES, sdO0 = sQ0 + C::BLK_BYTES;
+  const uint32_t vecs = sdO0 + C::BLK_BYTES;               // lse2[2][64], delta[2][64]
   const uint32_t bars = vecs + 2 * 2 * 64 * 4;
   const uint32_t bar_kv = bars, bar_s = bars + 8, bar_acc = bars + 16, bar_drain = bars + 24, bar_q0 = bars + 32;
   uint8_t* gen = smem_raw + (base - smem_u32(smem_raw));
@@ -711,14 +707,14 @@ __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_const
     mbar_init(bar_s, 1);
     mbar_init(bar_acc, 1);
     mbar_init(bar_drain, 1);
-    for (int s = 0; s < NST; ++s) mbar_init(bar_q0 + 8 * s, 1);
+    mbar_init(bar_q0, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tmRow);
     tma_prefetch_desc(&tmBlk);
     tma_prefetch_desc(&tmdO);
   }
   if (warp == 0) {
-    tmem_alloc(smem_u32(&tmem_base_smem), C::TCOLS_KV);
+    tmem_alloc(smem_u32(&tmem_base_smem), C::TCOLS);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -751,12 +747,11 @@ __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_const
   int fail = 0;
 
   auto load_q = [&](int j) {
-    const int st = (j - q0) % NST;
-    mbar_expect_tx(bar_q0 + 8 * st, 2 * C::BLK_BYTES);
+    mbar_expect_tx(bar_q0, 2 * C::BLK_BYTES);
 #pragma unroll
     for (int c = 0; c < C::NCH; ++c) {
-      tma_load_4d(sQ0 + st * C::BLK_BYTES + c * (TK * 128), &tmBlk, c * 64, h, j * TK, bs, bar_q0 + 8 * st);
-      tma_load_4d(sdO0 + st * C::BLK_BYTES + c * (TK * 128), &tmdO, c * 64, h, j * TK, nb, bar_q0 + 8 * st);
+      tma_load_4d(sQ0 + c * (TK * 128), &tmBlk, c * 64, h, j * TK, bs, bar_q0);
+      tma_load_4d(sdO0 + c * (TK * 128), &tmdO, c * 64, h, j * TK, nb, bar_q0);
     }
   };
   if (tid == 0) {
@@ -766,27 +761,21 @@ __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_const
       tma_load_4d(sK + c * (TQ * 128), &tmRow, c * 64, H + h, kb * TQ, bs, bar_kv);
       tma_load_4d(sV + c * (TQ * 128), &tmRow, c * 64, 2 * H + h, kb * TQ, bs, bar_kv);
     }
-    for (int i = 0; i < NST; ++i)
-      if (q0 + i < nq) load_q(q0 + i);
+    if (q0 < nq) load_q(q0);
   }
   const float c2 = scale * IL_LOG2E;
 
-  // S^T and dP^T of query block j; issued by thread 0 one step ahead (right after the previous block's dV/dK
-  // products) so that each sweep step waits for the tensor pipe only once
-  // descriptors of the operands at their first stage; a sweep step adds its stage's offset (one add per MMA:
-  // the issuing thread's own instruction stream is on every step's critical path)
+  // S^T and dP^T of query block j, issued by thread 0
   const SmemDescBase dk_k = make_smem_desc_base(sK, 16, 1024), dv_k = make_smem_desc_base(sV, 16, 1024);
   const SmemDescBase dq_k = make_smem_desc_base(sQ0, 16, 1024), ddo_k = make_smem_desc_base(sdO0, 16, 1024);
   const SmemDescBase dq_mn = make_smem_desc_base(sQ0, TK * 128, 1024), ddo_mn = make_smem_desc_base(sdO0, TK * 128, 1024);
   auto issue_s = [&](int j) {
-    const int it = j - q0, st = it % NST;
-    if (!mbar_wait(bar_q0 + 8 * st, (uint32_t)(it / NST) & 1u, abortp)) { fail = 1; abort_flag = 1; }
+    if (!mbar_wait(bar_q0, (uint32_t)(j - q0) & 1u, abortp)) { fail = 1; abort_flag = 1; }
     tc_fence_after();
-    const uint32_t so = (uint32_t)(st * C::BLK_BYTES);
 #pragma unroll
     for (int ks = 0; ks < DH / 16; ++ks) {
       const uint32_t off_a = (ks >> 2) * (TQ * 128) + (ks & 3) * 32;
-      const uint32_t off_b = so + (ks >> 2) * (TK * 128) + (ks & 3) * 32;
+      const uint32_t off_b = (ks >> 2) * (TK * 128) + (ks & 3) * 32;
       umma_bf16(tmem_base, desc_at(dk_k, off_a), desc_at(dq_k, off_b), idesc_s, ks ? 1u : 0u);
       if (PART != 1) umma_bf16(tmem_base + 64, desc_at(dv_k, off_a), desc_at(ddo_k, off_b), idesc_s, ks ? 1u : 0u);
     }
@@ -794,30 +783,20 @@ __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_const
   };
   if (tid == 0 && q0 < nq) {
     if (!mbar_wait(bar_kv, 0, abortp)) { fail = 1; abort_flag = 1; }
-    if (C::AHEAD) issue_s(q0);
   }
 
   for (int j = q0; j < nq; ++j) {
     const int it = j - q0;
-    const int st = it % NST;
     if (j + 1 < nq) put_vec(j + 1, vec_next);      // visible after this step's barrier
     vec_next = fetch_vec(j + 2);
-    if (!C::AHEAD) {
-      // single stage: the previous step's products must have retired before its tiles are replaced and the
-      // new scores overwrite the packed columns; only then are this step's scores issued
-      if (it > 0) {
-        if (!mbar_wait(bar_acc, (uint32_t)(it - 1) & 1u, abortp)) { fail = 1; abort_flag = 1; }
-        if (tid == 0) load_q(j);
-      }
-      if (tid == 0) issue_s(j);
+    // the previous step's products must have retired before its tiles are replaced and the new scores overwrite the packed
+    // columns; only then are this step's scores issued
+    if (it > 0) {
+      if (!mbar_wait(bar_acc, (uint32_t)(it - 1) & 1u, abortp)) { fail = 1; abort_flag = 1; }
+      if (tid == 0) load_q(j);
     }
+    if (tid == 0) issue_s(j);
     if (!mbar_wait(bar_s, (uint32_t)it & 1u, abortp)) { fail = 1; abort_flag = 1; }
-    // the previous step's dV/dK products were issued before these scores, so they have landed too: the packed
-    // P^T / dS^T columns and that step's Q/dO stage are free
-    // (the tensor pipe retires in order: bar_s covers them, only the last step's products are committed on their own)
-    if (C::AHEAD && it > 0) {
-      if (tid == 0 && j - 1 + NST < nq) load_q(j - 1 + NST);
-    }
     tc_fence_after();
     {
       float p[32], ds[32];
@@ -863,39 +842,34 @@ __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_const
     if (__syncthreads_or(fail)) { fail = 1; break; }
     if (tid == 0) {
       tc_fence_after();
-      const uint32_t so = (uint32_t)(st * C::BLK_BYTES);
 #pragma unroll
       for (int ks = 0; ks < TK / 16; ++ks) {
-        const uint32_t off_b = so + ks * 2048;                                              // MN-major: 16 queries
+        const uint32_t off_b = ks * 2048;                                                   // MN-major: 16 queries
         if (PART != 2)
           umma_bf16_ts(tmem_base + 128, tmem_base + packed_col(ks), desc_at(ddo_mn, off_b), idesc_g, (it | ks) ? 1u : 0u);
         if (PART != 1)
-          umma_bf16_ts(tmem_base + 128 + (PART == 0 ? DH : 0), tmem_base + 64 + packed_col(ks), desc_at(dq_mn, off_b), idesc_g,
+          umma_bf16_ts(tmem_base + 128, tmem_base + 64 + packed_col(ks), desc_at(dq_mn, off_b), idesc_g,
                        (it | ks) ? 1u : 0u);
       }
-      // every thread has read S^T / dP^T of this step (barrier above); the tensor pipe runs the products just
-      // issued, which read the packed columns, before it overwrites them with the next scores
-      if (C::AHEAD && j + 1 < nq) issue_s(j + 1);
-      else umma_commit(bar_acc);
+      umma_commit(bar_acc);
     }
   }
   const int nit = nq - q0;
   grid_dep_launch();
   if (!fail && nit > 0) {
-    if (!mbar_wait(bar_acc, C::AHEAD ? 0u : ((uint32_t)(nit - 1) & 1u), abortp)) { fail = 1; abort_flag = 1; }
+    if (!mbar_wait(bar_acc, (uint32_t)(nit - 1) & 1u, abortp)) { fail = 1; abort_flag = 1; }
     tc_fence_after();
   }
   fail = __syncthreads_or(fail);
   if (!fail) {
     bf16* rowp = dqkv + ((size_t)nb * T + key) * (3 * d) + h * DH;
     {
-      // one launch for both: the first half of the threads writes dV, the second half dK; a launch that holds
-      // one of them splits its columns between the two halves
-      const int which = PART == 0 ? hf : PART - 1;
-      const uint32_t tcol = t_lane + 128 + (PART == 0 ? which * DH : 0);
+      // the two halves of the threads split the columns
+      const int which = PART - 1;
+      const uint32_t tcol = t_lane + 128;
       bf16* dst = rowp + (which == 0 ? 2 * d : d);
       const float f = which == 0 ? 1.0f : scale;
-      const int cbeg = PART == 0 ? 0 : hf * (DH / 2), cend = PART == 0 ? DH : cbeg + DH / 2;
+      const int cbeg = hf * (DH / 2), cend = cbeg + DH / 2;
 #pragma unroll
       for (int c0 = cbeg; c0 < cend; c0 += 32) {
         float v[32];
@@ -936,7 +910,7 @@ __global__ void __launch_bounds__(256) attn_bwd_dkv_tc_kernel(const __grid_const
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, C::TCOLS_KV);
+    tmem_dealloc(tmem_base, C::TCOLS);
   }
 }
 
@@ -948,14 +922,13 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
                                                              bf16* __restrict__ dqkv, int B, int T, int H, float scale,
                                                              unsigned* err) {
   using C = BwdCfg<DH>;
-  constexpr int NST = C::NST;
   extern __shared__ uint8_t smem_raw[];
   __shared__ int abort_flag;
   __shared__ uint32_t tmem_base_smem;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sQ = base, sdO = sQ + C::ROW_BYTES;
-  const uint32_t sK0 = sdO + C::ROW_BYTES, sV0 = sK0 + NST * C::BLK_BYTES;
-  const uint32_t bars = sV0 + NST * C::BLK_BYTES;
+  const uint32_t sK0 = sdO + C::ROW_BYTES, sV0 = sK0 + C::BLK_BYTES;
+  const uint32_t bars = sV0 + C::BLK_BYTES;
   const uint32_t bar_q = bars, bar_s = bars + 8, bar_acc = bars + 16, bar_drain = bars + 24, bar_kv0 = bars + 32;
 
   // 256 threads: thread (r, hf) owns row r = tid % 128 and columns [32 hf, 32 hf + 32) of each 64-wide block
@@ -972,7 +945,7 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
   if (tid == 0) {
     abort_flag = 0;
     mbar_init(bar_q, 1);
-    for (int s = 0; s < NST; ++s) mbar_init(bar_kv0 + 8 * s, 1);
+    mbar_init(bar_kv0, 1);
     mbar_init(bar_s, 1);
     mbar_init(bar_acc, 1);
     mbar_init(bar_drain, 1);
@@ -982,7 +955,7 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
     tma_prefetch_desc(&tmdO);
   }
   if (warp == 0) {
-    tmem_alloc(smem_u32(&tmem_base_smem), C::TCOLS_Q);
+    tmem_alloc(smem_u32(&tmem_base_smem), C::TCOLS);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -997,12 +970,11 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
   int fail = 0;
 
   auto load_kv = [&](int j) {
-    const int st = j % NST;
-    mbar_expect_tx(bar_kv0 + 8 * st, 2 * C::BLK_BYTES);
+    mbar_expect_tx(bar_kv0, 2 * C::BLK_BYTES);
 #pragma unroll
     for (int c = 0; c < C::NCH; ++c) {
-      tma_load_4d(sK0 + st * C::BLK_BYTES + c * (TK * 128), &tmBlk, c * 64, H + h, j * TK, bs, bar_kv0 + 8 * st);
-      tma_load_4d(sV0 + st * C::BLK_BYTES + c * (TK * 128), &tmBlk, c * 64, 2 * H + h, j * TK, bs, bar_kv0 + 8 * st);
+      tma_load_4d(sK0 + c * (TK * 128), &tmBlk, c * 64, H + h, j * TK, bs, bar_kv0);
+      tma_load_4d(sV0 + c * (TK * 128), &tmBlk, c * 64, 2 * H + h, j * TK, bs, bar_kv0);
     }
   };
   if (tid == 0) {
@@ -1012,27 +984,23 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
       tma_load_4d(sQ + c * (TQ * 128), &tmRow, c * 64, h, qb * TQ, bs, bar_q);
       tma_load_4d(sdO + c * (TQ * 128), &tmdO, c * 64, h, qb * TQ, nb, bar_q);
     }
-    for (int i = 0; i < NST; ++i)
-      if (i < nkv) load_kv(i);
+    if (nkv > 0) load_kv(0);
   }
   const float c2 = scale * IL_LOG2E;
   const float lse2 = row < T ? lse[((size_t)bs * H + h) * T + row] * IL_LOG2E : 0.f;
   const float del = row < T ? delta[((size_t)nb * H + h) * T + row] : 0.f;
 
-  // S and dP of key block j; issued by thread 0 one step ahead (right after the previous block's dQ product)
-  // descriptors at the first stage; a sweep step adds its stage's offset (one add per MMA)
+  // S and dP of key block j, issued by thread 0
   const SmemDescBase dq_k = make_smem_desc_base(sQ, 16, 1024), ddo_k = make_smem_desc_base(sdO, 16, 1024);
   const SmemDescBase dk_k = make_smem_desc_base(sK0, 16, 1024), dv_k = make_smem_desc_base(sV0, 16, 1024);
   const SmemDescBase dk_mn = make_smem_desc_base(sK0, TK * 128, 1024);
   auto issue_s = [&](int j) {
-    const int st = j % NST;
-    if (!mbar_wait(bar_kv0 + 8 * st, (uint32_t)(j / NST) & 1u, abortp)) { fail = 1; abort_flag = 1; }
+    if (!mbar_wait(bar_kv0, (uint32_t)j & 1u, abortp)) { fail = 1; abort_flag = 1; }
     tc_fence_after();
-    const uint32_t so = (uint32_t)(st * C::BLK_BYTES);
 #pragma unroll
     for (int ks = 0; ks < DH / 16; ++ks) {
       const uint32_t off_a = (ks >> 2) * (TQ * 128) + (ks & 3) * 32;
-      const uint32_t off_b = so + (ks >> 2) * (TK * 128) + (ks & 3) * 32;
+      const uint32_t off_b = (ks >> 2) * (TK * 128) + (ks & 3) * 32;
       umma_bf16(tmem_base, desc_at(dq_k, off_a), desc_at(dk_k, off_b), idesc_s, ks ? 1u : 0u);
       umma_bf16(tmem_base + 64, desc_at(ddo_k, off_a), desc_at(dv_k, off_b), idesc_s, ks ? 1u : 0u);
     }
@@ -1040,22 +1008,16 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
   };
   if (tid == 0 && nkv > 0) {
     if (!mbar_wait(bar_q, 0, abortp)) { fail = 1; abort_flag = 1; }
-    if (C::AHEAD) issue_s(0);
   }
 
   for (int j = 0; j < nkv; ++j) {
-    const int st = j % NST;
-    if (!C::AHEAD) {      // single stage: retire the previous step's product, replace its tiles, then issue these scores
-      if (j > 0) {
-        if (!mbar_wait(bar_acc, (uint32_t)(j - 1) & 1u, abortp)) { fail = 1; abort_flag = 1; }
-        if (tid == 0) load_kv(j);
-      }
-      if (tid == 0) issue_s(j);
+    // retire the previous step's product, replace its tiles, then issue these scores
+    if (j > 0) {
+      if (!mbar_wait(bar_acc, (uint32_t)(j - 1) & 1u, abortp)) { fail = 1; abort_flag = 1; }
+      if (tid == 0) load_kv(j);
     }
+    if (tid == 0) issue_s(j);
     if (!mbar_wait(bar_s, (uint32_t)j & 1u, abortp)) { fail = 1; abort_flag = 1; }
-    if (C::AHEAD && j > 0) {                         // issued before these scores: landed (bar_s covers it), the packed dS and that step's K/V stage are free
-      if (tid == 0 && j - 1 + NST < nkv) load_kv(j - 1 + NST);
-    }
     tc_fence_after();
     {
       float ds[32];
@@ -1083,18 +1045,15 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
     if (__syncthreads_or(fail)) { fail = 1; break; }
     if (tid == 0) {
       tc_fence_after();
-      const uint32_t so = (uint32_t)(st * C::BLK_BYTES);
 #pragma unroll
       for (int ks = 0; ks < TK / 16; ++ks)
-        umma_bf16_ts(tmem_base + 128, tmem_base + 64 + packed_col(ks), desc_at(dk_mn, so + ks * 2048), idesc_g,
-                     (j | ks) ? 1u : 0u);
-      if (C::AHEAD && j + 1 < nkv) issue_s(j + 1);
-      else umma_commit(bar_acc);
+        umma_bf16_ts(tmem_base + 128, tmem_base + 64 + packed_col(ks), desc_at(dk_mn, ks * 2048), idesc_g, (j | ks) ? 1u : 0u);
+      umma_commit(bar_acc);
     }
   }
   grid_dep_launch();
   if (!fail && nkv > 0) {
-    if (!mbar_wait(bar_acc, C::AHEAD ? 0u : ((uint32_t)(nkv - 1) & 1u), abortp)) { fail = 1; abort_flag = 1; }
+    if (!mbar_wait(bar_acc, (uint32_t)(nkv - 1) & 1u, abortp)) { fail = 1; abort_flag = 1; }
     tc_fence_after();
   }
   fail = __syncthreads_or(fail);
@@ -1135,7 +1094,7 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, C::TCOLS_Q);
+    tmem_dealloc(tmem_base, C::TCOLS);
   }
 }
 
@@ -1676,44 +1635,44 @@ __global__ void __launch_bounds__(256) attn_delta_tc_kernel(const bf16* __restri
 }
 
 template <int DH>
+cudaError_t delta_launch(const bf16* dout, const bf16* o, float* delta, float* dq_zero, int NB, int B, int T, int H, cudaStream_t s) {
+  constexpr int TPR = (DH == 80) ? 16 : DH / 8;
+  const long long nthreads = (long long)NB * T * H * TPR;
+  return launch_dep(attn_delta_tc_kernel<DH>, dim3((unsigned)((nthreads + 255) / 256)), dim3(256), 0, s, dout, o, delta, dq_zero, NB, B, T, H);
+}
+
+template <int DH>
 cudaError_t bwd_tc_launch(const bf16* qkv, const bf16* o, const float* lse, const bf16* dout, bf16* dqkv, float* delta, int NB,
                           int B, int T, int H, unsigned* err, cudaStream_t s) {
-  using C = BwdCfg<DH>;
-  const unsigned long long d3 = 3ull * H * DH, d1 = (unsigned long long)H * DH;
-  const unsigned long long dims[4] = {(unsigned long long)DH, 3ull * H, (unsigned long long)T, (unsigned long long)B};
-  const unsigned long long strides[3] = {(unsigned long long)DH * 2, d3 * 2, (unsigned long long)T * d3 * 2};
-  const unsigned long long ddims[4] = {(unsigned long long)DH, (unsigned long long)H, (unsigned long long)T, (unsigned long long)NB};
-  const unsigned long long dstrides[3] = {(unsigned long long)DH * 2, d1 * 2, (unsigned long long)T * d1 * 2};
-  const unsigned box128[4] = {64, 1, TQ, 1}, box64[4] = {64, 1, TK, 1};
-  CUtensorMap tmRow, tmBlk, tmdO64, tmdO128;
-  if (!tma_encode_bf16(&tmRow, qkv, 4, dims, strides, box128) || !tma_encode_bf16(&tmBlk, qkv, 4, dims, strides, box64) ||
-      !tma_encode_bf16(&tmdO64, dout, 4, ddims, dstrides, box64) || !tma_encode_bf16(&tmdO128, dout, 4, ddims, dstrides, box128))
-    return cudaErrorInvalidValue;
-  constexpr bool SPLIT = 128 + 2 * DH > 512;      // dV and dK accumulators do not fit TMEM together: one launch each
-  cudaError_t e = cudaSuccess;
-  if constexpr (SPLIT) {
+  cudaError_t e = delta_launch<DH>(dout, o, delta, nullptr, NB, B, T, H, s);
+  if (e != cudaSuccess) return e;
+  if constexpr (DH <= 128) {
+    return attention_bwd_sweep(qkv, lse, dout, dqkv, delta, NB, B, T, H, DH, err, s);
+  } else {
+    using C = BwdCfg<DH>;
+    const unsigned long long d3 = 3ull * H * DH, d1 = (unsigned long long)H * DH;
+    const unsigned long long dims[4] = {(unsigned long long)DH, 3ull * H, (unsigned long long)T, (unsigned long long)B};
+    const unsigned long long strides[3] = {(unsigned long long)DH * 2, d3 * 2, (unsigned long long)T * d3 * 2};
+    const unsigned long long ddims[4] = {(unsigned long long)DH, (unsigned long long)H, (unsigned long long)T, (unsigned long long)NB};
+    const unsigned long long dstrides[3] = {(unsigned long long)DH * 2, d1 * 2, (unsigned long long)T * d1 * 2};
+    const unsigned box128[4] = {64, 1, TQ, 1}, box64[4] = {64, 1, TK, 1};
+    CUtensorMap tmRow, tmBlk, tmdO64, tmdO128;
+    if (!tma_encode_bf16(&tmRow, qkv, 4, dims, strides, box128) || !tma_encode_bf16(&tmBlk, qkv, 4, dims, strides, box64) ||
+        !tma_encode_bf16(&tmdO64, dout, 4, ddims, dstrides, box64) || !tma_encode_bf16(&tmdO128, dout, 4, ddims, dstrides, box128))
+      return cudaErrorInvalidValue;
     e = cudaFuncSetAttribute(attn_bwd_dkv_tc_kernel<DH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_KV);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(attn_bwd_dkv_tc_kernel<DH, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_KV);
-  } else {
-    e = cudaFuncSetAttribute(attn_bwd_dkv_tc_kernel<DH, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_KV);
-  }
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attn_bwd_dq_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_Q);
-  if (e != cudaSuccess) return e;
-  constexpr int TPR = (DH == 80) ? 16 : DH / 8;
-  const long long nthreads = (long long)NB * T * H * TPR;
-  launch_dep(attn_delta_tc_kernel<DH>, dim3((unsigned)((nthreads + 255) / 256)), dim3(256), 0, s, dout, o, delta, nullptr, NB, B, T, H);
-  dim3 grid((T + TQ - 1) / TQ, NB * H);
-  const float scale = rsqrtf((float)DH);
-  if constexpr (SPLIT) {
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(attn_bwd_dq_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_Q);
+    if (e != cudaSuccess) return e;
+    dim3 grid((T + TQ - 1) / TQ, NB * H);
+    const float scale = rsqrtf((float)DH);
     launch_dep(attn_bwd_dkv_tc_kernel<DH, 1>, dim3(grid), dim3(256), C::SMEM_KV, s, tmRow, tmBlk, tmdO64, lse, delta, dqkv, B, T, H, scale, err);
     launch_dep(attn_bwd_dkv_tc_kernel<DH, 2>, dim3(grid), dim3(256), C::SMEM_KV, s, tmRow, tmBlk, tmdO64, lse, delta, dqkv, B, T, H, scale, err);
-  } else {
-    launch_dep(attn_bwd_dkv_tc_kernel<DH, 0>, dim3(grid), dim3(256), C::SMEM_KV, s, tmRow, tmBlk, tmdO64, lse, delta, dqkv, B, T, H, scale, err);
+    launch_dep(attn_bwd_dq_tc_kernel<DH>, dim3(grid), dim3(256), C::SMEM_Q, s, tmRow, tmBlk, tmdO128, lse, delta, dqkv, B, T, H, scale, err);
+    return cudaGetLastError();
   }
-  launch_dep(attn_bwd_dq_tc_kernel<DH>, dim3(grid), dim3(256), C::SMEM_Q, s, tmRow, tmBlk, tmdO128, lse, delta, dqkv, B, T, H, scale, err);
-  return cudaGetLastError();
 }
 
 // One-sweep backward: delta (+ clearing the accumulator), the sweep, then dQ from fp32 to bf16.
@@ -1737,9 +1696,7 @@ cudaError_t bwd_fused_launch(const bf16* qkv, const bf16* o, const float* lse, c
   if (!tma_encode_f32(&tmAcc, dq_acc, 3, adims, astrides, abox)) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(attn_bwd_fused_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
-  constexpr int TPR = DH / 8;
-  const long long nthreads = (long long)NB * T * H * TPR;
-  launch_dep(attn_delta_tc_kernel<DH>, dim3((unsigned)((nthreads + 255) / 256)), dim3(256), 0, s, dout, o, delta, dq_acc, NB, B, T, H);
+  if ((e = delta_launch<DH>(dout, o, delta, dq_acc, NB, B, T, H, s)) != cudaSuccess) return e;
   // persistent CTAs, one per SM, each walking its share of the (key tile, sequence, head) items
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

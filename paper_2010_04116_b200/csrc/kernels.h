@@ -93,4 +93,8 @@ constexpr int ATTN_BWD_SHORT_T = 128;
 cudaError_t attention_bwd_short(const __nv_bfloat16* qkv, const float* lse, const __nv_bfloat16* dout, __nv_bfloat16* dqkv,
                                 int NB, int B, int T, int H, int dh, unsigned* err, cudaStream_t s);
 
+// dV, dK and dQ from qkv, lse, dout and delta, for head dimensions up to 128 (attention_sweep.cu); two kernels.
+cudaError_t attention_bwd_sweep(const __nv_bfloat16* qkv, const float* lse, const __nv_bfloat16* dout, __nv_bfloat16* dqkv,
+                                const float* delta, int NB, int B, int T, int H, int dh, unsigned* err, cudaStream_t s);
+
 }  // namespace il

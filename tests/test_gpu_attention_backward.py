@@ -1,5 +1,6 @@
-"""Attention backward of short sequences (one 128 x 128 tile): edges of the 16-wide contraction steps and of the two 64-key halves,
-more items than resident CTAs, every head dimension."""
+"""Attention backward with sums of fixed order, every head dimension: short sequences (one 128 x 128 tile) at the edges of the
+16-wide contraction steps and of the two 64-key halves, longer ones at the edges of the 128-row tiles and 64-wide sweep steps, more
+items than resident CTAs."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -11,8 +12,10 @@ DEV = "cuda:0"
 
 @pytest.mark.parametrize("dh", [32, 64, 80, 128, 256])
 @pytest.mark.parametrize("NB,B,T,H", [(1, 1, 2, 1), (2, 1, 15, 3), (2, 2, 16, 2), (4, 2, 17, 2), (3, 3, 63, 4), (2, 1, 64, 2), (2, 2, 65, 3),
-                                      (1, 1, 113, 2), (2, 1, 127, 2), (160, 80, 128, 4), (301, 301, 40, 1)])
-def test_short_backward_matches_fp64(NB, B, T, H, dh):
+                                      (1, 1, 113, 2), (2, 1, 127, 2), (160, 80, 128, 4), (301, 301, 40, 1),
+                                      (2, 1, 129, 2), (2, 2, 192, 1), (1, 1, 193, 3), (1, 1, 256, 2), (3, 1, 257, 2), (40, 20, 320, 4),
+                                      (2, 1, 1100, 3)])
+def test_backward_matches_fp64(NB, B, T, H, dh):
     g = torch.Generator(device=DEV)
     g.manual_seed(NB * T + dh)
     d = H * dh
@@ -30,13 +33,14 @@ def test_short_backward_matches_fp64(NB, B, T, H, dh):
     ref = torch.stack([ds @ k[idx], ds.transpose(-1, -2) @ q[idx], p.transpose(-1, -2) @ do])        # [3, NB, H, T, dh]
     ref = ref.permute(1, 3, 0, 2, 4).reshape(NB * T, 3 * d)
     got = torch.full((NB * T, 3 * d), 7.0, device=DEV, dtype=torch.bfloat16)
-    o = torch.zeros(B * T, d, device=DEV, dtype=torch.bfloat16)
+    o = (torch.softmax(s, -1) @ v).permute(0, 2, 1, 3).reshape(B * T, d).to(torch.bfloat16)
     delta = torch.zeros(NB * H * T, device=DEV)
     il.op_attention_bwd(qkv, o, lse.float(), dout, got, delta, NB, B, T, H, dh)
     torch.cuda.synchronize()
     for i in range(3):
         a, b = got[:, i * d:(i + 1) * d].double(), ref[:, i * d:(i + 1) * d]
-        # P or dS and the result are rounded to bf16, 2^-9 / sqrt(3) each in the mean: together 0.82 * 2^-9
+        # P or dS, the result and (in the row sums of longer sequences) O are rounded to bf16, 2^-9 / sqrt(3) each in the
+        # mean: together 2^-9
         assert float((a - b).norm() / b.norm()) < 2.0 ** -8, "qkv"[i]
     again = torch.full((NB * T, 3 * d), -3.0, device=DEV, dtype=torch.bfloat16)
     il.op_attention_bwd(qkv, o, lse.float(), dout, again, delta, NB, B, T, H, dh)
