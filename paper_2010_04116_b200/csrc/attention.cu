@@ -1099,42 +1099,49 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
 }
 
 // ------------------------------------------------------------------------------------------------
-// Backward in one sweep (head dimensions up to 64).  The two-kernel form above recomputes the scores twice (seven
+// Backward in one sweep (head dimensions up to 64).  The two-kernel forms recompute the scores twice (seven
 // products for five); here a CTA owns 128 keys, sweeps the queries in blocks of 128 and produces dV, dK and its
 // share of dQ from one recomputation of S^T and dP^T:
 //   S^T, dP^T   tcgen05.mma M128 (keys) N64 per 64-query half -> TMEM, two halves per step
-//   P^T, dS^T   threads (four per key row, 16 columns of a half each) recompute the probabilities from the saved
+//   P^T, dS^T   threads (two per key row and half, 32 columns each) recompute the probabilities from the saved
 //               log-sum-exp, round to bf16 and store the packed pairs back over the score columns
 //   dV += P^T dO, dK += dS^T Q      A operand read from those TMEM columns, accumulated over the whole sweep
 //   dQ_blk = dS K                   needs dS with the queries as rows: the same threads also write their dS values
 //                                   to shared memory in the layout of an MN-major A operand (swizzled 128-byte
 //                                   rows, one row per key); the product lands in one of two TMEM buffers and is
-//                                   added to an fp32 [rows, d] accumulator in global memory with red.add (every
+//                                   added to an fp32 [rows, d] accumulator in global memory by bulk reductions (every
 //                                   key tile of a (sequence, head) contributes to the same query rows)
-// Roles: warps 0-15 recompute and convert (four threads per key row), warps 16-19 add finished dQ blocks to the
-// global accumulator and store an item's dV / dK, warps 20 and 21 issue the MMAs (scores and dQ / dV and dK: a
-// single thread issues small MMAs no faster than one per ~54 cycles), warp 22 feeds the Q / dO ring by TMA and the
-// per-query lse / delta vectors by plain loads.  The halves
-// give the pipeline its overlap: while the threads work on one half of the step, the tensor pipe runs the other
-// half's products and the next step's scores for the half just finished.  One CTA per SM (all 512 TMEM columns,
-// ~195 KB of shared memory), persistent: a CTA walks a list of (key tile, sequence, head) items, and the loads and
-// scores of an item start while the previous item's dV / dK are still being written out.
+// Roles: warps 0-7 / 8-15 recompute and convert the first / second half of every step, warps 16-19 add finished dQ blocks to
+// the global accumulator, each its own 32 rows, and store an item's dV / dK, a thread each of warps 20, 21 and 22 issues the
+// MMAs of S and dV, of dP and dK, and of dQ, warp 23 feeds the Q / dO ring by TMA and the per-query lse / delta vectors by
+// plain loads.  The halves give the pipeline its overlap: while eight warps work on one half, the tensor pipe runs the other's
+// products and next scores.  One CTA per SM (all 512 TMEM columns, ~200 KB of shared memory), persistent: a CTA walks a list of
+// (key tile, sequence, head) items, and the loads and scores of an item start while the previous item's dV / dK are still
+// being written out.
+// What bounds it: a step of 128 x 128 takes about 3200 cycles, of which a recompute warp works 1400 (sixteen warps share the
+// issue slots) and an issuing thread 1700 (16 MMAs at 60, two commits at 120, looks at barriers at 150 each); the change of
+// items costs another step (K and V of one item only fit beside three Q / dO stages: with two buffers and two stages the tiles
+// came late and nothing was gained).  Measured, delta and conversion included: 16 x 16 heads x 1024, dh 64 236 -> 209 us, 8 x 16
+// 124 -> 107, against the form with all sixteen warps on either half in turn, one issuing thread per half and the four flush
+// warps staging a block together.
 // The sum over key tiles in dQ is made by floating-point atomics: its order, and with it the last bit of dQ,
 // depends on scheduling.  Every wait is bounded.
 // ------------------------------------------------------------------------------------------------
 template <int DH>
 struct FusedCfg {
   static constexpr int NST = 3;                          // Q / dO ring depth
+  static constexpr int KVB = 1;                          // items whose K / V are held (two would cost the ring a stage)
+  static constexpr int VST = 4;                          // ring of their lse / delta vectors, filled a step further ahead
   static constexpr int ROW_BYTES = TQ * 128;             // a 128-row operand (one 64-column chunk)
   static constexpr int DS_BYTES = 2 * TQ * 128;          // dS of one step: two 64-query chunks x 128 key rows x 128 B
   static constexpr int VEC_BYTES = 2 * TQ * 4;           // lse (log2 units) and delta of the step's 128 queries
-  static constexpr int SMEM = 2 * ROW_BYTES + NST * (2 * ROW_BYTES + VEC_BYTES) + 2 * DS_BYTES + 256 + 1024;
+  static constexpr int SMEM = KVB * 2 * ROW_BYTES + NST * 2 * ROW_BYTES + VST * VEC_BYTES + 2 * DS_BYTES + 256 + 1024;
   // TMEM columns: S^T [0,128) (two halves), dP^T [128,256), dV [256,256+DH), dK [320,320+DH), dQ [384,384+DH) / [448,448+DH)
   static constexpr int C_S = 0, C_DP = 128, C_DV = 256, C_DK = 320, C_DQ = 384;
 };
 
 constexpr int FUSED_THREADS = 768;   // warps 0-15 recompute, 16-19 flush dQ and store dV / dK, 20-22 issue MMAs, 23 loads
-constexpr int FUSED_RW = 16;         // recompute warps: four threads per key row, 16 query columns of a half each
+constexpr int FUSED_RW = 16;         // recompute warps: eight per half, two threads per key row, 32 query columns each
 
 // Work item = (key tile, gradient sequence, head).  Items are numbered key tile first, so the long sweeps (key tile
 // 0 sees every query block) come first; CTA c takes items c, c + gridDim.x, ...  Every role walks the same list and
@@ -1154,34 +1161,35 @@ __device__ __forceinline__ FusedItem fused_item(int item, int nbh, int H, int B,
 template <int DH>
 __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmRow,     // qkv, 128-row box
                                                                           const __grid_constant__ CUtensorMap tmdO,      // dout, 128-row box
-                                                                          const __grid_constant__ CUtensorMap tmAcc,     // dQ accumulator (fp32), 32 x 128 box
+                                                                          const __grid_constant__ CUtensorMap tmAcc,     // dQ accumulator (fp32), 32 x 32 box
                                                                           const float* __restrict__ lse, const float* __restrict__ delta,
                                                                           bf16* __restrict__ dqkv, int NB,
                                                                           int B, int T, int H, float scale, unsigned* err) {
   using C = FusedCfg<DH>;
-  constexpr int NST = C::NST;
+  constexpr int NST = C::NST, VST = C::VST, KVB = C::KVB;
   extern __shared__ uint8_t smem_raw[];
   __shared__ int abort_flag;
-  __shared__ volatile int flush_fail;
   __shared__ uint32_t tmem_base_smem;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t sK = base, sV = sK + C::ROW_BYTES;
-  const uint32_t sQ0 = sV + C::ROW_BYTES;                                  // stage st: Q at sQ0 + st * STAGE, dO after it
+  const uint32_t sKV = base;                                               // K of an item, V after it
+  const uint32_t sQ0 = sKV + KVB * 2 * C::ROW_BYTES;                             // stage st: Q at sQ0 + st * STAGE, dO after it
   constexpr uint32_t STAGE = 2 * C::ROW_BYTES;
   const uint32_t sDS = sQ0 + NST * STAGE;                                  // two dS buffers
-  const uint32_t sVec = sDS + 2 * C::DS_BYTES;                             // NST x (lse2[128], delta[128])
-  const uint32_t bars = sVec + NST * C::VEC_BYTES;
+  const uint32_t sVec = sDS + 2 * C::DS_BYTES;                             // VST x (lse2[128], delta[128])
+  const uint32_t bars = sVec + VST * C::VEC_BYTES;
   // barriers (8 bytes each)
-  const uint32_t bar_kv = bars, bar_kvfree = bars + 8, bar_acc = bars + 16, bar_accfree = bars + 24, bar_ds = bars + 32, bar_init = bars + 40;
-  auto bar_drain = [&](int t) { return bars + 48 + 8 * t; };                   // one per issuing thread
-  auto bar_full = [&](int st) { return bars + 72 + 8 * st; };
-  auto bar_empty = [&](int st) { return bars + 72 + 8 * (NST + st); };
-  auto bar_s = [&](int x) { return bars + 72 + 8 * (2 * NST + x); };           // scores of half x ready
-  auto bar_p = [&](int x) { return bars + 72 + 8 * (2 * NST + 2 + x); };       // P^T / dS^T of half x in tensor memory
-  auto bar_dq = [&](int b) { return bars + 72 + 8 * (2 * NST + 4 + b); };      // dQ buffer b complete
-  auto bar_dqfree = [&](int b) { return bars + 72 + 8 * (2 * NST + 6 + b); };  // dQ buffer b flushed
-  auto bar_vec = [&](int st) { return bars + 72 + 8 * (2 * NST + 8 + st); };   // lse / delta vectors of stage st written
-  auto bar_dsfree = [&](int b) { return bars + 72 + 8 * (3 * NST + 8 + b); };  // dS buffer b (also the staging of its dQ block) free again
+  auto bar_kv = [&](int i) { return bars + 8 * i; };                           // K / V buffer i loaded
+  auto bar_kvfree = [&](int i) { return bars + 16 + 8 * i; };
+  const uint32_t bar_acc = bars + 32, bar_accfree = bars + 40, bar_ds = bars + 48;
+  auto bar_drain = [&](int t) { return bars + 56 + 8 * t; };                   // one per issuing thread
+  auto bar_full = [&](int st) { return bars + 80 + 8 * st; };
+  auto bar_empty = [&](int st) { return bars + 80 + 8 * (NST + st); };
+  auto bar_s = [&](int x) { return bars + 80 + 8 * (2 * NST + x); };           // scores of half x ready
+  auto bar_p = [&](int x) { return bars + 80 + 8 * (2 * NST + 2 + x); };       // P^T / dS^T of half x in tensor memory
+  auto bar_dq = [&](int b) { return bars + 80 + 8 * (2 * NST + 4 + b); };      // dQ buffer b complete
+  auto bar_dqfree = [&](int b) { return bars + 80 + 8 * (2 * NST + 6 + b); };  // dQ buffer b flushed
+  auto bar_vec = [&](int v) { return bars + 80 + 8 * (2 * NST + 8 + v); };     // lse / delta vectors written
+  auto bar_dsfree = [&](int b) { return bars + 80 + 8 * (2 * NST + VST + 8 + b); };  // dS buffer b (also the staging of its dQ block) free again
   uint8_t* gen = smem_raw + (base - smem_u32(smem_raw));
   float* s_vec = reinterpret_cast<float*>(gen + (sVec - base));
 
@@ -1194,23 +1202,21 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
 
   if (tid == 0) {
     abort_flag = 0;
-    flush_fail = 0;
-    mbar_init(bar_kv, 1);
-    mbar_init(bar_kvfree, 3);            // the three issuing threads
-    mbar_init(bar_acc, 2);               // the two half threads
-    mbar_init(bar_init, 1);
+    for (int i = 0; i < 2; ++i) { mbar_init(bar_kv(i), 1); mbar_init(bar_kvfree(i), 3); }    // (freed by the three issuing threads)
+    mbar_init(bar_acc, 2);               // the threads of dV and of dK
     mbar_init(bar_accfree, 4);           // one arrival per flush warp
     mbar_init(bar_ds, FUSED_RW);         // one arrival per recompute warp
     mbar_init(bar_drain(0), 1);
     mbar_init(bar_drain(1), 1);
     mbar_init(bar_drain(2), 1);
-    for (int st = 0; st < NST; ++st) { mbar_init(bar_full(st), 1); mbar_init(bar_empty(st), 2); mbar_init(bar_vec(st), 1); }
+    for (int st = 0; st < NST; ++st) { mbar_init(bar_full(st), 1); mbar_init(bar_empty(st), 2); }
+    for (int v = 0; v < VST; ++v) mbar_init(bar_vec(v), 1);
     for (int x = 0; x < 2; ++x) {
-      mbar_init(bar_s(x), 1);
-      mbar_init(bar_p(x), FUSED_RW);
+      mbar_init(bar_s(x), 2);            // the threads of S and of dP
+      mbar_init(bar_p(x), FUSED_RW / 2);
       mbar_init(bar_dq(x), 1);
       mbar_init(bar_dqfree(x), 4);       // one arrival per flush warp
-      mbar_init(bar_dsfree(x), 1);
+      mbar_init(bar_dsfree(x), 4);       // (likewise)
     }
     fence_mbar_init();
     tma_prefetch_desc(&tmRow);
@@ -1231,114 +1237,131 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
 
   if (warp == 23) {
     // ---------------------------------------------------------------- loads
+    // lse (log2 units) and delta of a step's queries, by plain loads: into registers two steps ahead of the tiles, into shared
+    // memory one step ahead.  Slot of step g + 1 = slot of step g - NST, whose readers are done: the stage of that step was
+    // waited for.
+    static_assert(VST == NST + 1, "a slot is free when the tiles of the step before its next use are requested");
+    int v_item = blockIdx.x, v_it = 0, v_g = 0;
+    float v_lse[4], v_del[4];
+    auto fetch_vectors = [&]() {
+      if (v_item >= nitems) return;
+      const FusedItem w = fused_item(v_item, nbh, H, B, nq);
+      const float* lse_b = lse + ((size_t)w.bs * H + w.h) * T;
+      const float* del_b = delta + ((size_t)w.nb * H + w.h) * T;
+#pragma unroll
+      for (int q4 = 0; q4 < 4; ++q4) {
+        const int q = (w.kb + v_it) * TQ + q4 * 32 + lane;
+        v_lse[q4] = q < T ? lse_b[q] : 0.f;
+        v_del[q4] = q < T ? del_b[q] : 0.f;
+      }
+    };
+    auto put_vectors = [&]() {                                   // ... and the next ones are asked for
+      if (v_item >= nitems) return;
+      float* vec = s_vec + (v_g % VST) * (2 * TQ);
+#pragma unroll
+      for (int q4 = 0; q4 < 4; ++q4) {
+        vec[q4 * 32 + lane] = v_lse[q4] * IL_LOG2E;
+        vec[TQ + q4 * 32 + lane] = v_del[q4];
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_vec(v_g % VST));            // its release publishes the warp's stores
+      ++v_g;
+      if (++v_it == fused_item(v_item, nbh, H, B, nq).nit) { v_it = 0; v_item += gridDim.x; }
+      fetch_vectors();
+    };
+    fetch_vectors();
+    put_vectors();
     int g = 0, n_item = 0;
     for (int item = blockIdx.x; item < nitems && !fail; item += gridDim.x, ++n_item) {
       const FusedItem w = fused_item(item, nbh, H, B, nq);
-      const float* lse_b = lse + ((size_t)w.bs * H + w.h) * T;
-      const float* del_b = delta + ((size_t)w.nb * H + w.h) * T;
       for (int it = 0; it < w.nit; ++it) {
         const int gs = g + it, st = gs % NST, j = w.kb + it;
         int ok = 1;
         if (lane == 0 && gs >= NST) ok = mbar_wait(bar_empty(st), (uint32_t)(gs / NST - 1) & 1u, abortp) ? 1 : 0;
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) { fail = 1; abort_flag = 1; break; }
-        // the tiles first (their latency is the longer one), then the step's lse / delta vectors by plain loads,
-        // published on a barrier of their own
         if (lane == 0) {
           mbar_expect_tx(bar_full(st), 2 * C::ROW_BYTES);
           tma_load_4d(sQ0 + st * STAGE, &tmRow, 0, w.h, j * TQ, w.bs, bar_full(st));
           tma_load_4d(sQ0 + st * STAGE + C::ROW_BYTES, &tmdO, 0, w.h, j * TQ, w.nb, bar_full(st));
         }
-        float* vec = s_vec + st * (2 * TQ);
-#pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4) {
-          const int q = j * TQ + q4 * 32 + lane;
-          vec[q4 * 32 + lane] = q < T ? lse_b[q] * IL_LOG2E : 0.f;
-          vec[TQ + q4 * 32 + lane] = q < T ? del_b[q] : 0.f;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_vec(st));                   // its release publishes the warp's stores
         if (it == 0) {
-          // the item's K and V (after its first query block, which does not depend on the previous item): their
-          // buffers are free once the previous item's last products that read them have retired
+          // the item's K and V: their buffer is free once the previous item's last products that read them have retired
           int ok2 = 1;
-          if (lane == 0 && n_item > 0) ok2 = mbar_wait(bar_kvfree, (uint32_t)(n_item - 1) & 1u, abortp) ? 1 : 0;
+          const int kb = n_item % KVB;
+          if (lane == 0 && n_item >= KVB) ok2 = mbar_wait(bar_kvfree(kb), (uint32_t)(n_item / KVB - 1) & 1u, abortp) ? 1 : 0;
           ok2 = __shfl_sync(0xffffffffu, ok2, 0);
           if (!ok2) { fail = 1; abort_flag = 1; break; }
           if (lane == 0) {
-            mbar_expect_tx(bar_kv, 2 * C::ROW_BYTES);
-            tma_load_4d(sK, &tmRow, 0, H + w.h, w.kb * TQ, w.bs, bar_kv);
-            tma_load_4d(sV, &tmRow, 0, 2 * H + w.h, w.kb * TQ, w.bs, bar_kv);
+            mbar_expect_tx(bar_kv(kb), 2 * C::ROW_BYTES);
+            tma_load_4d(sKV + kb * STAGE, &tmRow, 0, H + w.h, w.kb * TQ, w.bs, bar_kv(kb));
+            tma_load_4d(sKV + kb * STAGE + C::ROW_BYTES, &tmRow, 0, 2 * H + w.h, w.kb * TQ, w.bs, bar_kv(kb));
           }
         }
+        put_vectors();
       }
       g += w.nit;
     }
     grid_dep_launch();
   } else if (warp == 20 || warp == 21) {
-    // ---------------------------------------------------------------- MMA issue, one thread per half x of the query block
-    // A thread issues small MMAs no faster than one per ~54 cycles, and every hand-over between threads costs a
-    // commit / barrier round trip of several hundred cycles.  So each half has its own issuing thread that does, in
-    // program order (the tensor pipe keeps one thread's MMAs in order), dV += P^T(x) dO(x), dK += dS^T(x) Q(x) and
-    // then the next step's S^T(x), dP^T(x) into the score columns those products have just read.  Both threads add
-    // into the same dV / dK accumulators (the pipe executes one MMA at a time; the order in which the two halves are
-    // added is not fixed).
+    // ---------------------------------------------------------------- MMA issue: S and dV, dP and dK
+    // A thread issues small MMAs no faster than one per ~60 cycles, a commit costs it 120, a look at a barrier 150, and every
+    // hand-over between threads a round trip of several hundred.  One thread does S and dV, the other dP and dK: in program
+    // order (the tensor pipe keeps one thread's MMAs in order) a half's product and then the next step's scores of that half,
+    // into the columns the product has just read.  Each accumulator belongs to one thread, so its sums have a fixed order.
     if (lane == 0) {
       const int x = warp - 20;
       constexpr uint32_t idesc_s = make_idesc_bf16(TQ, TK, 0, 0);          // S^T / dP^T half: M128 N64, both K-major
       constexpr uint32_t idesc_g = make_idesc_bf16(TQ, DH, 0, 1);          // dV / dK: A from TMEM, B MN-major
-      const SmemDescBase dk_k = make_smem_desc_base(sK, 16, 1024), dv_k = make_smem_desc_base(sV, 16, 1024);
-      const SmemDescBase dq_k = make_smem_desc_base(sQ0, 16, 1024), ddo_k = make_smem_desc_base(sQ0 + C::ROW_BYTES, 16, 1024);
-      const SmemDescBase dq_mn = make_smem_desc_base(sQ0, TQ * 128, 1024), ddo_mn = make_smem_desc_base(sQ0 + C::ROW_BYTES, TQ * 128, 1024);
+      const SmemDescBase rows = make_smem_desc_base(sKV + (x ? C::ROW_BYTES : 0), 16, 1024);             // K / V
+      const SmemDescBase cols = make_smem_desc_base(sQ0 + (x ? C::ROW_BYTES : 0), 16, 1024);             // Q / dO
+      const SmemDescBase other = make_smem_desc_base(sQ0 + (x ? 0 : C::ROW_BYTES), TQ * 128, 1024);      // dO / Q
+      const uint32_t t_s = tmem_base + (x ? C::C_DP : C::C_S), t_acc = tmem_base + (x ? C::C_DK : C::C_DV);
       bool ok = true;
-      // scores of this half of the step held in stage st: rows 64x .. 64x+63 of the Q / dO tiles (8 KB further)
-      auto issue_scores = [&](int st) {
-        const uint32_t so = (uint32_t)st * STAGE + (uint32_t)x * (TK * 128);
+      // scores of half hf of the step held in stage st: rows 64 hf .. 64 hf + 63 of its tile (8 KB further)
+      auto issue_scores = [&](int hf, int st, int kb) {
+        const uint32_t so = (uint32_t)st * STAGE + (uint32_t)hf * (TK * 128), ko = (uint32_t)kb * STAGE;
 #pragma unroll
-        for (int ks = 0; ks < DH / 16; ++ks) {
-          umma_bf16(tmem_base + C::C_S + 64 * x, desc_at(dk_k, ks * 32), desc_at(dq_k, so + ks * 32), idesc_s, ks ? 1u : 0u);
-          umma_bf16(tmem_base + C::C_DP + 64 * x, desc_at(dv_k, ks * 32), desc_at(ddo_k, so + ks * 32), idesc_s, ks ? 1u : 0u);
-        }
-        umma_commit(bar_s(x));
+        for (int ks = 0; ks < DH / 16; ++ks)
+          umma_bf16(t_s + 64 * hf, desc_at(rows, ko + ks * 32), desc_at(cols, so + ks * 32), idesc_s, ks ? 1u : 0u);
+        umma_commit(bar_s(hf));
       };
       int g = 0, n_item = 0;
       for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++n_item) {
         const FusedItem w = fused_item(item, nbh, H, B, nq);
+        const int kb = n_item % KVB;
         // first step of the item: its scores need the item's K / V and the step's Q / dO (the score columns are free:
         // this thread's own last products of the previous item come before them in the pipe)
-        if (!mbar_wait(bar_kv, (uint32_t)n_item & 1u, abortp)) { ok = false; break; }
+        if (!mbar_wait(bar_kv(kb), (uint32_t)(n_item / KVB) & 1u, abortp)) { ok = false; break; }
         if (!mbar_wait(bar_full(g % NST), (uint32_t)(g / NST) & 1u, abortp)) { ok = false; break; }
         tc_fence_after();
-        issue_scores(g % NST);
-        // the accumulators still hold the previous item's dV / dK until they have been stored; the half-1 thread also
-        // lets the half-0 thread's first products (which overwrite instead of adding) go first
+        issue_scores(0, g % NST, kb);
+        issue_scores(1, g % NST, kb);
+        // the accumulator still holds the previous item's dV / dK until it has been stored
         if (n_item > 0 && !mbar_wait(bar_accfree, (uint32_t)(n_item - 1) & 1u, abortp)) { ok = false; break; }
-        if (x == 1 && !mbar_wait(bar_init, (uint32_t)n_item & 1u, abortp)) { ok = false; break; }
         for (int it = 0; it < w.nit && ok; ++it) {
           const int gs = g + it, st = gs % NST, st1 = (gs + 1) % NST;
           const uint32_t ph = (uint32_t)gs & 1u;
           const bool more = it + 1 < w.nit;
-          if (!mbar_wait(bar_p(x), ph, abortp)) { ok = false; break; }
-          tc_fence_after();
-          // dV += P^T(x) dO(x), dK += dS^T(x) Q(x): contraction over the half's 64 queries (MN-major B: 16 queries = 2048 B)
-          const uint32_t so = (uint32_t)st * STAGE + (uint32_t)x * (TK * 128);
 #pragma unroll
-          for (int ks = 0; ks < TK / 16; ++ks) {
-            const uint32_t acc = (it | x | ks) ? 1u : 0u;
-            umma_bf16_ts(tmem_base + C::C_DV, tmem_base + C::C_S + 64 * x + 16 * ks, desc_at(ddo_mn, so + ks * 2048), idesc_g, acc);
-            umma_bf16_ts(tmem_base + C::C_DK, tmem_base + C::C_DP + 64 * x + 16 * ks, desc_at(dq_mn, so + ks * 2048), idesc_g, acc);
-          }
-          if (x == 0 && it == 0) umma_commit(bar_init);
-          umma_commit(bar_empty(st));                       // (one of two arrivals) the stage's tiles have been read by this half
-          if (more) {
-            if (!mbar_wait(bar_full(st1), (uint32_t)((gs + 1) / NST) & 1u, abortp)) { ok = false; break; }
+          for (int hf = 0; hf < 2; ++hf) {
+            if (!mbar_wait(bar_p(hf), ph, abortp)) { ok = false; break; }
             tc_fence_after();
-            issue_scores(st1);
-          } else {
-            umma_commit(bar_kvfree);                        // (one of three) nothing of this item reads K / V from this thread any more
-            umma_commit(bar_acc);                           // (one of two) this half's share of dV / dK is complete
+            // dV += P^T dO / dK += dS^T Q: contraction over the half's 64 queries (MN-major B: 16 queries = 2048 B)
+            const uint32_t so = (uint32_t)st * STAGE + (uint32_t)hf * (TK * 128);
+#pragma unroll
+            for (int ks = 0; ks < TK / 16; ++ks)
+              umma_bf16_ts(t_acc, t_s + 64 * hf + packed_col(ks), desc_at(other, so + ks * 2048), idesc_g, (it | hf | ks) ? 1u : 0u);
+            if (hf == 1) umma_commit(bar_empty(st));          // (one of two arrivals) this thread's products have read the stage
+            if (more) {
+              if (hf == 0 && !mbar_wait(bar_full(st1), (uint32_t)((gs + 1) / NST) & 1u, abortp)) { ok = false; break; }
+              issue_scores(hf, st1, kb);
+            }
           }
         }
+        if (!ok) break;
+        umma_commit(bar_kvfree(kb));                          // (one of three) nothing of this item reads K / V from this thread any more
+        umma_commit(bar_acc);                                 // (one of two) dV / dK is complete
         g += w.nit;
       }
       if (!ok) { fail = 1; abort_flag = 1; }
@@ -1350,13 +1373,15 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
     // ---------------------------------------------------------------- MMA issue, third thread: dQ
     if (lane == 0) {
       constexpr uint32_t idesc_q = make_idesc_bf16(TQ, DH, 1, 1);          // A = dS (MN-major), B = K (MN-major)
-      const SmemDescBase dk_mn = make_smem_desc_base(sK, TQ * 128, 1024);
+      const SmemDescBase dk_mn = make_smem_desc_base(sKV, TQ * 128, 1024);
       const SmemDescBase dds_mn = make_smem_desc_base(sDS, TQ * 128, 1024);
       bool ok = true;
       int g = 0, n_item = 0;
       for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++n_item) {
         const FusedItem w = fused_item(item, nbh, H, B, nq);
-        if (!mbar_wait(bar_kv, (uint32_t)n_item & 1u, abortp)) { ok = false; break; }     // this item's K is in place
+        const int kb = n_item % KVB;
+        const uint32_t ko = (uint32_t)kb * STAGE;
+        if (!mbar_wait(bar_kv(kb), (uint32_t)(n_item / KVB) & 1u, abortp)) { ok = false; break; }     // this item's K is in place
         for (int it = 0; it < w.nit && ok; ++it) {
           const int gs = g + it, b = gs & 1;
           // dQ(step) = dS K over this tile's 128 keys: both halves of dS are in shared memory (bar_ds; the item's K
@@ -1367,10 +1392,10 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
           tc_fence_after();
 #pragma unroll
           for (int ks = 0; ks < TQ / 16; ++ks)
-            umma_bf16(tmem_base + C::C_DQ + 64 * b, desc_at(dds_mn, (uint32_t)b * C::DS_BYTES + ks * 2048), desc_at(dk_mn, ks * 2048),
+            umma_bf16(tmem_base + C::C_DQ + 64 * b, desc_at(dds_mn, (uint32_t)b * C::DS_BYTES + ks * 2048), desc_at(dk_mn, ko + ks * 2048),
                       idesc_q, ks ? 1u : 0u);
           umma_commit(bar_dq(b));
-          if (it + 1 == w.nit) umma_commit(bar_kvfree);      // (one of three)
+          if (it + 1 == w.nit) umma_commit(bar_kvfree(kb));      // (one of three)
         }
         g += w.nit;
       }
@@ -1383,63 +1408,11 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
     // ---------------------------------------------------------------- dQ flush and dV / dK store (warps 16-19: thread = row)
     const int r = tid - 512;
     const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-    // The four flush warps meet at a named barrier inside every step, so they must leave the loops together: the
-    // outcome of a wait is agreed on (through a shared flag and that barrier) before anyone acts on it.
-    auto all_ok = [&](int got) -> bool {
-      if (!got) flush_fail = 1;
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      return flush_fail == 0;
-    };
-    int g = 0, n_item = 0;
-    for (int item = blockIdx.x; item < nitems && !fail; item += gridDim.x, ++n_item) {
-      const FusedItem w = fused_item(item, nbh, H, B, nq);
-      for (int it = 0; it < w.nit; ++it) {
-        const int gs = g + it, b = gs & 1;
-        int got = 1;
-        if (lane == 0) got = mbar_wait(bar_dq(b), (uint32_t)(gs >> 1) & 1u, abortp) ? 1 : 0;
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (!all_ok(got)) { fail = 1; abort_flag = 1; break; }
-        tc_fence_after();
-        // The block goes to the global accumulator as one bulk reduction per 32 columns: the rows are staged in the
-        // dS buffer of this step (its dQ product, the only reader, has retired) in the 128-byte-swizzled layout of
-        // the tensor map, and one thread issues cp.reduce.async.bulk.tensor (rows past the sequence end are dropped
-        // by the map's bounds).
-        const uint32_t stage = sDS + (uint32_t)b * C::DS_BYTES;
-#pragma unroll
-        for (int c0 = 0; c0 < DH; c0 += 32) {
-          uint32_t rr[32];
-          tmem_ld_32x32(t_lane + C::C_DQ + 64 * b + c0, rr);
-          tmem_ld_wait();
-          const uint32_t rowaddr = stage + (uint32_t)(c0 / 32) * (TQ * 128) + (uint32_t)r * 128;
-#pragma unroll
-          for (int t = 0; t < 8; ++t)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rowaddr + (((uint32_t)t ^ (uint32_t)(r & 7)) * 16)), "r"(rr[4 * t]),
-                         "r"(rr[4 * t + 1]), "r"(rr[4 * t + 2]), "r"(rr[4 * t + 3])
-                         : "memory");
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_dqfree(b));               // the TMEM buffer has been read
-        fence_proxy_async();
-        asm volatile("bar.sync 1, 128;" ::: "memory");           // the four flush warps: the block is staged
-        if (r == 0) {
-#pragma unroll
-          for (int c0 = 0; c0 < DH; c0 += 32)
-            tma_reduce_add_3d(&tmAcc, stage + (uint32_t)(c0 / 32) * (TQ * 128), w.h * DH + c0, (w.kb + it) * TQ, w.nb);
-          bulk_commit_group();
-          bulk_wait_group_read0();                               // the staging has been read: the buffer may be rewritten
-          mbar_arrive(bar_dsfree(b));
-        }
-      }
-      if (fail) break;
-      g += w.nit;
-      // the item's dV and dK: this thread's key row, scaled and rounded to bf16
-      {
-        int got = 1;
-        if (lane == 0) got = mbar_wait(bar_acc, (uint32_t)n_item & 1u, abortp) ? 1 : 0;
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (!all_ok(got)) { fail = 1; abort_flag = 1; break; }
-      }
+    // (a warp's rows are its own throughout: waits, staging and reductions need no meeting of the four)
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abortp)); };
+    // an item's dV and dK: this thread's key row, scaled and rounded to bf16
+    auto store_item = [&](const FusedItem& w, int n_item) -> bool {
+      if (!wait(bar_acc, (uint32_t)n_item & 1u)) return false;
       tc_fence_after();
       const int key = w.kb * TQ + r;
       bf16* rowp = dqkv + ((size_t)w.nb * T + key) * (3 * d) + w.h * DH;
@@ -1469,90 +1442,131 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_accfree);               // the accumulators may be overwritten by the next item
+      return true;
+    };
+    int g = 0, n_item = 0;
+    for (int item = blockIdx.x; item < nitems && !fail; item += gridDim.x, ++n_item) {
+      const FusedItem w = fused_item(item, nbh, H, B, nq);
+      for (int it = 0; it < w.nit; ++it) {
+        const int gs = g + it, b = gs & 1;
+        // (before the last dQ block: the next item's first products wait for the accumulators)
+        if (it + 1 == w.nit && !store_item(w, n_item)) { fail = 1; abort_flag = 1; break; }
+        if (!wait(bar_dq(b), (uint32_t)(gs >> 1) & 1u)) { fail = 1; abort_flag = 1; break; }
+        tc_fence_after();
+        // The warp's 32 rows go to the global accumulator as one bulk reduction per 32 columns: they are staged in the dS
+        // buffer of this step (its dQ product, the only reader, has retired) in the 128-byte-swizzled layout of the tensor
+        // map, and one thread issues cp.reduce.async.bulk.tensor (rows past the sequence end are dropped by the map's bounds).
+        const uint32_t stage = sDS + (uint32_t)b * C::DS_BYTES;
+#pragma unroll
+        for (int c0 = 0; c0 < DH; c0 += 32) {
+          uint32_t rr[32];
+          tmem_ld_32x32(t_lane + C::C_DQ + 64 * b + c0, rr);
+          tmem_ld_wait();
+          const uint32_t rowaddr = stage + (uint32_t)(c0 / 32) * (TQ * 128) + (uint32_t)r * 128;
+#pragma unroll
+          for (int t = 0; t < 8; ++t)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rowaddr + (((uint32_t)t ^ (uint32_t)(r & 7)) * 16)), "r"(rr[4 * t]),
+                         "r"(rr[4 * t + 1]), "r"(rr[4 * t + 2]), "r"(rr[4 * t + 3])
+                         : "memory");
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_dqfree(b));               // the TMEM buffer has been read
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+          const int row0 = (w.kb + it) * TQ + (warp & 3) * 32;
+          if (row0 < T) {
+#pragma unroll
+            for (int c0 = 0; c0 < DH; c0 += 32)
+              tma_reduce_add_3d(&tmAcc, stage + (uint32_t)(c0 / 32) * (TQ * 128) + (uint32_t)(warp & 3) * (32 * 128), w.h * DH + c0, row0, w.nb);
+          }
+          bulk_commit_group();
+          bulk_wait_group_read0();                               // the staging has been read: the buffer may be rewritten
+          mbar_arrive(bar_dsfree(b));
+        }
+        __syncwarp();
+      }
+      if (fail) break;
+      g += w.nit;
     }
-    if (r == 0) bulk_wait_group0();                            // every reduction this thread issued has reached memory
+    if (lane == 0) bulk_wait_group0();                         // every reduction this thread issued has reached memory
   } else if (warp < FUSED_RW) {
     // ---------------------------------------------------------------- recompute and convert (warps 0-15)
-    // thread (r, sub): key row r, query columns [16 sub, 16 sub + 16) of each 64-column half
-    const int r = tid & 127, sub = tid >> 7;
+    // Warps 0-7 take the first half of every step, 8-15 the second; thread = key row r, query columns 32 hc .. 32 hc + 31 of
+    // the half.
+    const int x = warp >> 3, hc = (warp >> 2) & 1, r = tid & 127;
     const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-    auto wait = [&](uint32_t bar, uint32_t parity) -> bool {     // lane 0 polls, the warp learns the outcome
-      int got = 1;
-      if (lane == 0) got = mbar_wait(bar, parity, abortp) ? 1 : 0;
-      return __shfl_sync(0xffffffffu, got, 0) != 0;
+    const uint32_t t_s = t_lane + C::C_S + 64 * x + 32 * hc, t_dp = t_lane + C::C_DP + 64 * x + 32 * hc;
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+      return __all_sync(0xffffffffu, mbar_wait(bar, parity, abortp));
     };
     int g = 0;
     for (int item = blockIdx.x; item < nitems && !fail; item += gridDim.x) {
       const FusedItem w = fused_item(item, nbh, H, B, nq);
       const int key = w.kb * TQ + r;
-      for (int it = 0; it < w.nit && !fail; ++it) {
-        const int gs = g + it, st = gs % NST, b = gs & 1, j = w.kb + it;
-        const uint32_t ph = (uint32_t)gs & 1u;
-        const float* vec = s_vec + st * (2 * TQ);
-        // the stage's lse / delta vectors have their own barrier; the dS buffer of this step is free once the dQ
-        // block of step gs-2, staged in it after its product, has been handed to the bulk reduction
-        if (!wait(bar_vec(st), (uint32_t)(gs / NST) & 1u)) { fail = 1; abort_flag = 1; break; }
-        if (gs >= 2 && !wait(bar_dsfree(b), (uint32_t)((gs >> 1) - 1) & 1u)) { fail = 1; abort_flag = 1; break; }
-        const bool diag = (it == 0);                       // some queries of this block precede some keys of this tile
-        const bool tail = (j * TQ + TQ > T);
-        for (int x = 0; x < 2; ++x) {
-          if (!wait(bar_s(x), ph)) { fail = 1; abort_flag = 1; break; }
-          tc_fence_after();
-          uint32_t r0[16], r1[16];
-          tmem_ld_32x16(t_lane + C::C_S + 64 * x + 16 * sub, r0);
-          tmem_ld_32x16(t_lane + C::C_DP + 64 * x + 16 * sub, r1);
+      for (int it = 0; it < w.nit; ++it) {
+        const int gs = g + it, b = gs & 1, j = w.kb + it;
+        const float4* lv = reinterpret_cast<const float4*>(s_vec + (gs % VST) * (2 * TQ) + 64 * x + 32 * hc);
+        const float4* dv_ = reinterpret_cast<const float4*>(s_vec + (gs % VST) * (2 * TQ) + TQ + 64 * x + 32 * hc);
+        if (!wait(bar_vec(gs % VST), (uint32_t)(gs / VST) & 1u) || !wait(bar_s(x), (uint32_t)gs & 1u)) { fail = 1; abort_flag = 1; break; }
+        tc_fence_after();
+        const bool masked = it == 0 || j * TQ + TQ > T;    // uniform: some queries precede some keys, or lie past the sequence
+        const int qbase = j * TQ + 64 * x + 32 * hc;
+        uint32_t dw[16];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {                      // 16 columns at a time: the register budget of 768 threads
+          uint32_t s[16], dp[16], pw[8], dc[8];
+          tmem_ld_32x16(t_s + 16 * c, s);
+          tmem_ld_32x16(t_dp + 16 * c, dp);
           tmem_ld_wait();
-          float p[16], ds[16];
-          const float4* lv = reinterpret_cast<const float4*>(vec + 64 * x + 16 * sub);
-          const float4* dv_ = reinterpret_cast<const float4*>(vec + TQ + 64 * x + 16 * sub);
-          const int qbase = j * TQ + 64 * x + 16 * sub;
+          float p[16];
 #pragma unroll
-          for (int i4 = 0; i4 < 4; ++i4) {
-            const float4 l4 = lv[i4], d4 = dv_[i4];
-            const float ll[4] = {l4.x, l4.y, l4.z, l4.w}, dd[4] = {d4.x, d4.y, d4.z, d4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int i = 4 * i4 + e;
-              p[i] = ex2_fast(fmaf(__uint_as_float(r0[i]), c2, -ll[e]));
-              ds[i] = __uint_as_float(r1[i]) - dd[e];
-            }
+          for (int i = 0; i < 16; i += 4) {
+            const float4 l = lv[4 * c + i / 4];
+            p[i] = ex2_fast(fmaf(__uint_as_float(s[i]), c2, -l.x));
+            p[i + 1] = ex2_fast(fmaf(__uint_as_float(s[i + 1]), c2, -l.y));
+            p[i + 2] = ex2_fast(fmaf(__uint_as_float(s[i + 2]), c2, -l.z));
+            p[i + 3] = ex2_fast(fmaf(__uint_as_float(s[i + 3]), c2, -l.w));
           }
-          if (diag || tail) {                              // uniform across the CTA
+          if (masked) {
 #pragma unroll
             for (int i = 0; i < 16; ++i)
-              if (qbase + i < key || qbase + i >= T) p[i] = 0.f;
+              if (qbase + 16 * c + i < key || qbase + 16 * c + i >= T) p[i] = 0.f;
           }
-          uint32_t pw[8], dw[8];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            pw[i] = pack_bf16x2(p[2 * i], p[2 * i + 1]);
-            dw[i] = pack_bf16x2(ds[2 * i] * p[2 * i], ds[2 * i + 1] * p[2 * i + 1]);
+          for (int i = 0; i < 16; i += 4) {
+            const float4 e = dv_[4 * c + i / 4];
+            dc[i / 2] = pack_bf16x2((__uint_as_float(dp[i]) - e.x) * p[i], (__uint_as_float(dp[i + 1]) - e.y) * p[i + 1]);
+            dc[i / 2 + 1] = pack_bf16x2((__uint_as_float(dp[i + 2]) - e.z) * p[i + 2], (__uint_as_float(dp[i + 3]) - e.w) * p[i + 3]);
+            pw[i / 2] = pack_bf16x2(p[i], p[i + 1]);
+            pw[i / 2 + 1] = pack_bf16x2(p[i + 2], p[i + 3]);
           }
-          tmem_st_32x8(t_lane + C::C_S + 64 * x + 16 * sub, pw);      // P^T over the first half of the columns this thread read
-          tmem_st_32x8(t_lane + C::C_DP + 64 * x + 16 * sub, dw);     // dS^T likewise
-          tmem_st_wait();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_p(x));                       // dV / dK of this half can go
-          // dS as the A operand of dQ = dS K: row = key, 64 queries of half x = one swizzled 128-byte row of chunk x
-          {
-            const uint32_t rowaddr = sDS + (uint32_t)b * C::DS_BYTES + (uint32_t)x * (TQ * 128) + (uint32_t)r * 128;
+          tmem_st_32x8(t_s + 8 * c, pw);                   // P^T over columns this thread has read
+          tmem_st_32x8(t_dp + 8 * c, dc);                  // dS^T likewise
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-              const uint32_t unit = (uint32_t)(2 * sub + t) ^ (uint32_t)(r & 7);
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rowaddr + unit * 16), "r"(dw[4 * t]), "r"(dw[4 * t + 1]),
-                           "r"(dw[4 * t + 2]), "r"(dw[4 * t + 3])
-                           : "memory");
-            }
-          }
-          if (x == 1) {
-            fence_proxy_async();                             // both halves' dS rows are read by the tensor pipe (async proxy)
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_ds);
-          }
+          for (int i = 0; i < 8; ++i) dw[8 * c + i] = dc[i];
         }
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_p(x));              // dV / dK of this half can go
+        // dS as the A operand of dQ = dS K: row = key, 64 queries of half x = one swizzled 128-byte row of chunk x.  Its
+        // buffer is free once the dQ block of step gs-2, staged in it after its product, has been handed to the bulk reduction.
+        if (gs >= 2 && !wait(bar_dsfree(b), (uint32_t)((gs >> 1) - 1) & 1u)) { fail = 1; abort_flag = 1; break; }
+        const uint32_t rowaddr = sDS + (uint32_t)b * C::DS_BYTES + (uint32_t)x * (TQ * 128) + (uint32_t)r * 128;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const uint32_t unit = (uint32_t)(4 * hc + t) ^ (uint32_t)(r & 7);
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rowaddr + unit * 16), "r"(dw[4 * t]), "r"(dw[4 * t + 1]),
+                       "r"(dw[4 * t + 2]), "r"(dw[4 * t + 3])
+                       : "memory");
+        }
+        fence_proxy_async();                               // the dS rows are read by the tensor pipe (async proxy)
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_ds);
       }
-      if (fail) break;
       g += w.nit;
     }
   }
@@ -1689,10 +1703,10 @@ cudaError_t bwd_fused_launch(const bf16* qkv, const bf16* o, const float* lse, c
   CUtensorMap tmRow, tmdO, tmAcc;
   if (!tma_encode_bf16(&tmRow, qkv, 4, dims, strides, box128) || !tma_encode_bf16(&tmdO, dout, 4, ddims, dstrides, box128))
     return cudaErrorInvalidValue;
-  // the fp32 dQ accumulator [NB, T, d] as the target of the bulk reductions: boxes of 32 columns x 128 rows of one sequence
+  // the fp32 dQ accumulator [NB, T, d] as the target of the bulk reductions: boxes of 32 columns x 32 rows of one sequence
   const unsigned long long adims[3] = {d1, (unsigned long long)T, (unsigned long long)NB};
   const unsigned long long astrides[2] = {d1 * 4, (unsigned long long)T * d1 * 4};
-  const unsigned abox[3] = {32, TQ, 1};
+  const unsigned abox[3] = {32, 32, 1};
   if (!tma_encode_f32(&tmAcc, dq_acc, 3, adims, astrides, abox)) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(attn_bwd_fused_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
