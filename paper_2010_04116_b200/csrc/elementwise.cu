@@ -372,34 +372,42 @@ cudaError_t layernorm_bwd_rows(const void* dy, int dy_is_f32, const float* x, co
 }
 
 // ---------------------------------------------------------------------------------------------
-// LayerNorm backward in one pass over the rows (bf16 dy, d = 128 NV with NV <= 8): the row part as above and, for
+// LayerNorm backward in one pass over the rows (bf16 dy, d up to 4096): the row part as above and, for
 // the rows of the first gradient stream (row < x_rows), the column reductions that otherwise take three more
 // kernels over the same data: dgamma += dy * xhat, dbeta += dy, and colsum += the kernel's own output (the bias
-// gradient of the linear layer whose output this residual-stream gradient belongs to).  A warp walks rows with a
-// grid-wide stride, keeps a row's values in registers between the two passes and its column partials in
-// registers across rows; the block combines its eight warps through shared memory and adds one value per
-// column and output to global memory.  dgamma / dbeta / colsum must be zeroed (or hold a sum to add to).
+// gradient of the linear layer whose output this residual-stream gradient belongs to).  W warps (one up to d 1024, two, four)
+// walk rows with a grid-wide stride, keep a row's values in registers between the two passes (NV float4 a lane and array) and
+// their column partials in registers across rows; the block combines its warps through shared memory and adds one value
+// per column and output to global memory.  dgamma / dbeta / colsum must be zeroed (or hold a sum to add to).
+// TAIL: the width is not W NV 128, the last columns of the layout are empty.
+// What bounds it: the bytes (dy, x, residual in, dx and its bf16 copy out).  Widths beyond 1024 and those that are no multiple of
+// 128 took four kernels (row part, parameter sums, and a bias gradient's column sums over 42 MB at 4096 x 2560 that were read
+// again): a step of 2.7B widths 11.7 -> 11.35 ms.
 // ---------------------------------------------------------------------------------------------
-template <int NV>
+template <int NV, int W, bool TAIL>
 __global__ void __launch_bounds__(256, 1) layernorm_bwd_fused_kernel(const bf16* __restrict__ dy, const float* __restrict__ x,
                                                                      const float* __restrict__ mean,
                                                                      const float* __restrict__ rstd,
                                                                      const float* __restrict__ gamma, const float* resid,
                                                                      float* dx_out, bf16* __restrict__ dx_bf16,
                                                                      float* __restrict__ dgamma, float* __restrict__ dbeta,
-                                                                     float* __restrict__ colsum, int rows, int x_rows) {
+                                                                     float* __restrict__ colsum, int rows, int x_rows, int d_arg) {
   grid_dep_wait();
-  constexpr int d = NV * 128;
+  const int d = TAIL ? d_arg : NV * 128 * W;
   __shared__ float4 red[8][NV * 32];
+  __shared__ float2 part[2][8];                   // a row's two sums by warp, rows in turn
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int warps = gridDim.x * 8;
+  const int team = w / W, first_col = (w % W) * (NV * 32) + lane;
+  auto in = [&](int i) { return !TAIL || first_col + 32 * i < (d >> 2); };
+  const int teams = gridDim.x * (8 / W);
+  int turn = 0;
   float4 g4[NV];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) g4[i] = __ldg(reinterpret_cast<const float4*>(gamma) + lane + 32 * i);
+  for (int i = 0; i < NV; ++i) g4[i] = in(i) ? __ldg(reinterpret_cast<const float4*>(gamma) + first_col + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
   float4 ag[NV], ab[NV], ac[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) ag[i] = ab[i] = ac[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int row = blockIdx.x * 8 + w; row < rows; row += warps) {
+  for (int row = blockIdx.x * (8 / W) + team; row < rows; row += teams) {
     const int xrow = row % x_rows;
     const bool first = row < x_rows;              // rows of the first stream feed the parameter gradients
     const float mu = mean[xrow], rs = rstd[xrow];
@@ -408,8 +416,10 @@ __global__ void __launch_bounds__(256, 1) layernorm_bwd_fused_kernel(const bf16*
     float s1 = 0.f, s2 = 0.f;
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      dv[i] = load_dy4<false>(dy, (size_t)row, d, lane + 32 * i);
-      const float4 xv = xr[lane + 32 * i];
+      dv[i] = xh[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (!in(i)) continue;
+      dv[i] = load_dy4<false>(dy, (size_t)row, d, first_col + 32 * i);
+      const float4 xv = xr[first_col + 32 * i];
       xh[i] = make_float4((xv.x - mu) * rs, (xv.y - mu) * rs, (xv.z - mu) * rs, (xv.w - mu) * rs);
     }
 #pragma unroll
@@ -422,30 +432,42 @@ __global__ void __launch_bounds__(256, 1) layernorm_bwd_fused_kernel(const bf16*
         ab[i].x += dv[i].x; ab[i].y += dv[i].y; ab[i].z += dv[i].z; ab[i].w += dv[i].w;
       }
     }
-    const float m1 = warp_sum(s1) / d;
-    const float m2 = warp_sum(s2) / d;          // mean of dxhat * xhat
+    s1 = warp_sum(s1);
+    s2 = warp_sum(s2);
+    if constexpr (W > 1) {                        // the team's sums, added in warp order
+      if (lane == 0) part[turn][w] = make_float2(s1, s2);
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(32 * W) : "memory");
+      s1 = s2 = 0.f;
+#pragma unroll
+      for (int k = 0; k < W; ++k) { const float2 t = part[turn][team * W + k]; s1 += t.x; s2 += t.y; }
+      turn ^= 1;                                  // (the next row's sums go elsewhere; the one after comes past that row's barrier)
+    }
+    const float m1 = s1 / d;
+    const float m2 = s2 / d;                    // mean of dxhat * xhat
     const float4* rr = resid ? reinterpret_cast<const float4*>(resid + (size_t)row * d) : nullptr;
     float4* outr = reinterpret_cast<float4*>(dx_out + (size_t)row * d);
     uint2* outb = dx_bf16 ? reinterpret_cast<uint2*>(dx_bf16 + (size_t)row * d) : nullptr;
     float4 r4[NV];
     if (rr) {
 #pragma unroll
-      for (int i = 0; i < NV; ++i) r4[i] = rr[lane + 32 * i];
+      for (int i = 0; i < NV; ++i)
+        if (in(i)) r4[i] = rr[first_col + 32 * i];
     }
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
+      if (!in(i)) continue;
       float4 o;
       o.x = (dv[i].x * g4[i].x - m1 - xh[i].x * m2) * rs;
       o.y = (dv[i].y * g4[i].y - m1 - xh[i].y * m2) * rs;
       o.z = (dv[i].z * g4[i].z - m1 - xh[i].z * m2) * rs;
       o.w = (dv[i].w * g4[i].w - m1 - xh[i].w * m2) * rs;
       if (rr) { o.x += r4[i].x; o.y += r4[i].y; o.z += r4[i].z; o.w += r4[i].w; }
-      outr[lane + 32 * i] = o;
+      outr[first_col + 32 * i] = o;
       if (outb) {
         uint2 b;
         b.x = pack_bf16x2(o.x, o.y);
         b.y = pack_bf16x2(o.z, o.w);
-        outb[lane + 32 * i] = b;
+        outb[first_col + 32 * i] = b;
       }
       if (first) { ac[i].x += o.x; ac[i].y += o.y; ac[i].z += o.z; ac[i].w += o.w; }
     }
@@ -459,11 +481,13 @@ __global__ void __launch_bounds__(256, 1) layernorm_bwd_fused_kernel(const bf16*
 #pragma unroll
     for (int i = 0; i < NV; ++i) red[w][lane + 32 * i] = q == 0 ? ag[i] : q == 1 ? ab[i] : ac[i];
     __syncthreads();
-    for (int c = threadIdx.x; c < NV * 32; c += 256) {
-      float4 t = red[0][c];
+    for (int c = threadIdx.x; c < NV * 32 * W; c += 256) {
+      if (TAIL && 4 * c >= d) break;
+      const int wr = c / (NV * 32), at = c - wr * (NV * 32);
+      float4 t = red[wr][at];
 #pragma unroll
-      for (int k = 1; k < 8; ++k) {
-        const float4 v = red[k][c];
+      for (int k = 1; k < 8 / W; ++k) {
+        const float4 v = red[k * W + wr][at];
         t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
       }
       red_add_f32x4(out + 4 * c, t);
@@ -472,24 +496,24 @@ __global__ void __launch_bounds__(256, 1) layernorm_bwd_fused_kernel(const bf16*
   }
 }
 
-// Fused LayerNorm backward for bf16 dy when d is a multiple of 128 up to 1024; returns cudaErrorNotSupported for
-// other widths (the caller then uses the separate row and column kernels).  dgamma, dbeta, colsum: fp32 [d],
-// summed into (colsum may be NULL).
+// Fused LayerNorm backward for bf16 dy and d a multiple of four up to 4096; returns cudaErrorNotSupported for other widths (the
+// caller then uses the separate row and column kernels).  dgamma, dbeta, colsum: fp32 [d], summed into (colsum may be NULL).
 cudaError_t layernorm_bwd_fused(const bf16* dy, const float* x, const float* mean, const float* rstd, const float* gamma,
                                 const float* resid, float* dx_out, bf16* dx_bf16, float* dgamma, float* dbeta,
                                 float* colsum, int rows, int x_rows, int d, cudaStream_t s) {
-  if (d % 128 || d > 1024 || d < 128) return cudaErrorNotSupported;
-  int blocks = ceil_div(rows, 8);
+  if (d % 4 || d > LN_BWD_FUSED_MAX || d < 4) return cudaErrorNotSupported;
+  const int W = d <= 1024 ? 1 : d <= 2048 ? 2 : 4, nv = ceil_div(d, 128 * W);
+  const bool tail = d != nv * 128 * W;
+  int blocks = ceil_div(rows, 8 / W);
   if (blocks > 148) blocks = 148;
-#define IL_LNF(NV)                                                                                                        \
-  case NV:                                                                                                                \
-    launch_dep(layernorm_bwd_fused_kernel<NV>, dim3(blocks), dim3(256), 0, s, dy, x, mean, rstd, gamma, resid, dx_out, dx_bf16, dgamma, dbeta, \
-                                                          colsum, rows, x_rows);                                          \
-    break;
-  switch (d / 128) {
-    IL_LNF(1) IL_LNF(2) IL_LNF(3) IL_LNF(4) IL_LNF(5) IL_LNF(6) IL_LNF(7) IL_LNF(8)
-  }
-#undef IL_LNF
+#define IL_LNF1(NV, W_)                                                                                                  \
+  if (nv == NV && W == W_)                                                                                               \
+    launch_dep(tail ? layernorm_bwd_fused_kernel<NV, W_, true> : layernorm_bwd_fused_kernel<NV, W_, false>, dim3(blocks), dim3(256), 0, s, dy, \
+               x, mean, rstd, gamma, resid, dx_out, dx_bf16, dgamma, dbeta, colsum, rows, x_rows, d);
+  IL_LNF1(1, 1) IL_LNF1(2, 1) IL_LNF1(3, 1) IL_LNF1(4, 1) IL_LNF1(5, 1) IL_LNF1(6, 1) IL_LNF1(7, 1) IL_LNF1(8, 1)
+  IL_LNF1(5, 2) IL_LNF1(6, 2) IL_LNF1(7, 2) IL_LNF1(8, 2)
+  IL_LNF1(5, 4) IL_LNF1(6, 4) IL_LNF1(7, 4) IL_LNF1(8, 4)
+#undef IL_LNF1
   return cudaGetLastError();
 }
 

@@ -33,7 +33,8 @@ cudaError_t layernorm_bwd_rows(const void* dy, int dy_is_f32, const float* x, co
 // Outputs are accumulated atomically and must be zeroed by the caller.
 cudaError_t layernorm_bwd_params(const void* dy, int dy_is_f32, const float* x, const float* mean, const float* rstd,
                                  float* dgamma, float* dbeta, int rows, int d, cudaStream_t s);
-// Both of the above in one pass for bf16 dy and d a multiple of 128 up to 1024 (cudaErrorNotSupported otherwise),
+constexpr int LN_BWD_FUSED_MAX = 4096;
+// Both of the above in one pass for bf16 dy and d a multiple of 4 up to LN_BWD_FUSED_MAX (cudaErrorNotSupported otherwise),
 // plus, when colsum != NULL, colsum[c] += sum over the first x_rows rows of dx_out[r,c].
 cudaError_t layernorm_bwd_fused(const __nv_bfloat16* dy, const float* x, const float* mean, const float* rstd,
                                 const float* gamma, const float* resid, float* dx_out, __nv_bfloat16* dx_bf16, float* dgamma,

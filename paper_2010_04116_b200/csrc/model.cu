@@ -1180,7 +1180,7 @@ il_status layers_backward(il_model* m, int k, int s, size_t base, int count, con
   const int N = m->ntok, d = m->d, F = m->F;
   const int R = s * N;
   CompScratch& c = m->cs[k];
-  const bool fused_ln = d % 128 == 0 && d <= 1024;     // widths the one-pass LayerNorm backward covers
+  const bool fused_ln = d <= LN_BWD_FUSED_MAX;         // widths the one-pass LayerNorm backward covers
   BackwardBranch br(m, k, R, F);
   for (int l = count - 1; l >= 0; --l) {
     const LayerOff& o = m->layer_off[base + l];
