@@ -382,7 +382,7 @@ cudaError_t layernorm_bwd_rows(const void* dy, int dy_is_f32, const float* x, co
 // TAIL: the width is not W NV 128, the last columns of the layout are empty.
 // What bounds it: the bytes (dy, x, residual in, dx and its bf16 copy out).  Widths beyond 1024 and those that are no multiple of
 // 128 took four kernels (row part, parameter sums, and a bias gradient's column sums over 42 MB at 4096 x 2560 that were read
-// again): a step of 2.7B widths 11.7 -> 11.35 ms.
+// again): a step of 2.7B widths 11.7 -> 11.35 ms for a few steps, 12.26 -> 12.15 under the power cap.
 // ---------------------------------------------------------------------------------------------
 template <int NV, int W, bool TAIL>
 __global__ void __launch_bounds__(256, 1) layernorm_bwd_fused_kernel(const bf16* __restrict__ dy, const float* __restrict__ x,
