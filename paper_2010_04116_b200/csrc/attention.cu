@@ -1177,19 +1177,29 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
   const uint32_t sDS = sQ0 + NST * STAGE;                                  // two dS buffers
   const uint32_t sVec = sDS + 2 * C::DS_BYTES;                             // VST x (lse2[128], delta[128])
   const uint32_t bars = sVec + VST * C::VEC_BYTES;
-  // barriers (8 bytes each)
-  auto bar_kv = [&](int i) { return bars + 8 * i; };                           // K / V buffer i loaded
-  auto bar_kvfree = [&](int i) { return bars + 16 + 8 * i; };
-  const uint32_t bar_acc = bars + 32, bar_accfree = bars + 40, bar_ds = bars + 48;
-  auto bar_drain = [&](int t) { return bars + 56 + 8 * t; };                   // one per issuing thread
-  auto bar_full = [&](int st) { return bars + 80 + 8 * st; };
-  auto bar_empty = [&](int st) { return bars + 80 + 8 * (NST + st); };
-  auto bar_s = [&](int x) { return bars + 80 + 8 * (2 * NST + x); };           // scores of half x ready
-  auto bar_p = [&](int x) { return bars + 80 + 8 * (2 * NST + 2 + x); };       // P^T / dS^T of half x in tensor memory
-  auto bar_dq = [&](int b) { return bars + 80 + 8 * (2 * NST + 4 + b); };      // dQ buffer b complete
-  auto bar_dqfree = [&](int b) { return bars + 80 + 8 * (2 * NST + 6 + b); };  // dQ buffer b flushed
-  auto bar_vec = [&](int v) { return bars + 80 + 8 * (2 * NST + 8 + v); };     // lse / delta vectors written
-  auto bar_dsfree = [&](int b) { return bars + 80 + 8 * (2 * NST + VST + 8 + b); };  // dS buffer b (also the staging of its dQ block) free again
+  // Barriers (8 bytes each).  A wait by parity is right only while the phase before the awaited one is over and the one after it
+  // cannot be; and a phase of several arrivals must not collect those of two steps.  Every waiter below waits for all phases of a
+  // barrier in turn, and after each barrier stands what holds its next phase back until all have passed this one.
+  auto bar_kv = [&](int i) { return bars + 8 * i; };                           // K / V buffer i loaded: the loader waits for bar_kvfree
+  auto bar_kvfree = [&](int i) { return bars + 16 + 8 * i; };                  // arrivals follow bar_kv, which the loader lets go
+  const uint32_t bar_acc = bars + 32;                                          // dV / dK complete: next products wait for bar_accfree
+  const uint32_t bar_accfree = bars + 40;                                      // ... stored: arrivals follow bar_acc
+  // dS of a step written by both halves, into buffer b.  One per buffer: the halves run up to a step apart, so a barrier for
+  // both buffers would count the faster half's next step in the slower one's stead.  Arrivals at this buffer's next
+  // step follow bar_dsfree(b).
+  auto bar_ds = [&](int b) { return bars + 48 + 8 * b; };
+  auto bar_drain = [&](int t) { return bars + 64 + 8 * t; };                   // one per issuing thread, used once
+  auto bar_full = [&](int st) { return bars + 88 + 8 * st; };                  // Q / dO of a step loaded: the loader waits for bar_empty
+  auto bar_empty = [&](int st) { return bars + 88 + 8 * (NST + st); };         // arrivals follow bar_full
+  auto bar_s = [&](int x) { return bars + 88 + 8 * (2 * NST + x); };           // scores of half x ready: each issuing thread waits for bar_p(x)
+  auto bar_p = [&](int x) { return bars + 88 + 8 * (2 * NST + 2 + x); };       // P^T / dS^T of half x in tensor memory: arrivals follow bar_s(x)
+  auto bar_dq = [&](int b) { return bars + 88 + 8 * (2 * NST + 4 + b); };      // dQ buffer b complete: its thread waits for bar_dqfree(b)
+  auto bar_dqfree = [&](int b) { return bars + 88 + 8 * (2 * NST + 6 + b); };  // dQ buffer b flushed: arrivals follow bar_dq(b)
+  auto bar_vec = [&](int v) { return bars + 88 + 8 * (2 * NST + 8 + v); };     // lse / delta vectors written: the loader has waited for bar_empty of
+                                                                               // the slot's last step, which follows all reads of it
+  auto bar_dsfree = [&](int b) { return bars + 88 + 8 * (2 * NST + VST + 8 + b); };  // dS buffer b (also the staging of its dQ block) free
+                                                                               // again: arrivals follow bar_dq(b), which follows bar_ds(b)
+  static_assert(88 + 8 * (2 * C::NST + C::VST + 10) <= 256, "barriers");
   uint8_t* gen = smem_raw + (base - smem_u32(smem_raw));
   float* s_vec = reinterpret_cast<float*>(gen + (sVec - base));
 
@@ -1205,7 +1215,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
     for (int i = 0; i < 2; ++i) { mbar_init(bar_kv(i), 1); mbar_init(bar_kvfree(i), 3); }    // (freed by the three issuing threads)
     mbar_init(bar_acc, 2);               // the threads of dV and of dK
     mbar_init(bar_accfree, 4);           // one arrival per flush warp
-    mbar_init(bar_ds, FUSED_RW);         // one arrival per recompute warp
+    for (int b = 0; b < 2; ++b) mbar_init(bar_ds(b), FUSED_RW);     // one arrival per recompute warp
     mbar_init(bar_drain(0), 1);
     mbar_init(bar_drain(1), 1);
     mbar_init(bar_drain(2), 1);
@@ -1387,7 +1397,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
           // dQ(step) = dS K over this tile's 128 keys: both halves of dS are in shared memory (bar_ds; the item's K
           // arrived before the scores that dS came from), buffer b of the accumulator is free once the flush of
           // step gs-2 is done
-          if (!mbar_wait(bar_ds, (uint32_t)gs & 1u, abortp)) { ok = false; break; }
+          if (!mbar_wait(bar_ds(b), (uint32_t)(gs >> 1) & 1u, abortp)) { ok = false; break; }
           if (gs >= 2 && !mbar_wait(bar_dqfree(b), (uint32_t)((gs >> 1) - 1) & 1u, abortp)) { ok = false; break; }
           tc_fence_after();
 #pragma unroll
@@ -1565,7 +1575,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) attn_bwd_fused_kernel(const 
         }
         fence_proxy_async();                               // the dS rows are read by the tensor pipe (async proxy)
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_ds);
+        if (lane == 0) mbar_arrive(bar_ds(b));
       }
       g += w.nit;
     }

@@ -46,3 +46,40 @@ def test_backward_matches_fp64(NB, B, T, H, dh):
     il.op_attention_bwd(qkv, o, lse.float(), dout, again, delta, NB, B, T, H, dh)
     torch.cuda.synchronize()
     assert torch.equal(got, again)                # every sum has a fixed order
+
+
+@pytest.mark.parametrize("dh", [32, 64])
+@pytest.mark.parametrize("NB,B,T,H", [(40, 20, 320, 4), (3, 3, 257, 60), (16, 8, 501, 16), (151, 151, 129, 1), (2, 1, 2049, 12)])
+def test_one_sweep_with_several_items_per_cta(NB, B, T, H, dh):
+    """More (key tile, sequence, head) items than SMs, of several lengths: K / V, accumulators, rings and step counters go from
+    item to item.  Against the fixed-order form (above against fp64): dK and dV bit for bit, dQ, whose share of every key tile
+    has the same bits there and here, up to the order of their fp32 sum and one rounding to bf16."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(NB + T + dh)
+    d = H * dh
+    qkv = torch.randn(B * T, 3 * d, device=DEV, generator=g).to(torch.bfloat16)
+    dout = torch.randn(NB * T, d, device=DEV, generator=g).to(torch.bfloat16)
+    o, lse = torch.empty(B * T, d, device=DEV, dtype=torch.bfloat16), torch.empty(B, H, T, device=DEV)
+    il.op_attention_fwd(qkv, o, lse, B, T, H, dh)
+    delta, acc = torch.empty(NB * H * T, device=DEV), torch.full((NB * T, d), 9.0, device=DEV)
+    two = torch.empty(NB * T, 3 * d, device=DEV, dtype=torch.bfloat16)
+    il.op_attention_bwd(qkv, o, lse, dout, two, delta, NB, B, T, H, dh)
+    err = torch.zeros(1, dtype=torch.int32, device=DEV)
+    one = torch.empty_like(two)
+    a = torch.randn(1024, 1024, device=DEV, dtype=torch.bfloat16)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    for attempt in range(6):
+        one.fill_(5.0)
+        if attempt % 2:                           # beside kernels of another stream
+            with torch.cuda.stream(side):
+                for _ in range(20):
+                    a @ a
+        il.op_attention_bwd_one_sweep(qkv, o, lse, dout, one, delta, acc, NB, B, T, H, dh, err_word=err)
+        torch.cuda.synchronize()
+        assert int(err.item()) == 0
+        assert torch.equal(one[:, d:], two[:, d:])
+        x, y = (t[:, :d].float().view(NB, T, H, dh).permute(0, 2, 1, 3) for t in (one, two))
+        for t0 in range(0, T, 128):               # tile by tile: one that missed a share is not lost among the others
+            num, den = ((x - y)[:, :, t0:t0 + 128].norm(dim=(-1, -2)), y[:, :, t0:t0 + 128].norm(dim=(-1, -2)))
+            assert bool((num <= 2.0 ** -8 * den).all()), (attempt, t0)
