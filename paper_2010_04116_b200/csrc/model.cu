@@ -1259,8 +1259,8 @@ il_status head_backward(il_model* m, int k, bool acc, float scale) {
   // the GPU idle on small batches, is planned as one of (at least) two that run side by side
   const int beside = m->placement == IL_PLACE_SINGLE && m->K > 1 ? 2 : 1;
   BackwardBranch br(m, k, N, d);
+  IL_TRY(br.fork());              // (the branch is joined below whether or not this pass gives it work)
   if (!acc) {   // vectors are summed into atomically; embedding rows no token selects must read zero
-    IL_TRY(br.fork());
     IL_CUDA(m, cudaMemsetAsync(m->G[k] + m->comp_mat_end[k], 0, (m->comp_end[k] - m->comp_mat_end[k]) * 4, br.st));
     if (k == 0) {
       IL_CUDA(m, cudaMemsetAsync(m->G[k] + m->off_wte, 0, (size_t)V * d * 4, br.st));

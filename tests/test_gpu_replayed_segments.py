@@ -60,3 +60,20 @@ def test_replay_after_the_rule_and_window_change():
                 for x, y in zip(seen[n, rule], r):
                     assert np.array_equal(x, y)
             seen.setdefault((n, rule), r)
+
+
+def test_recompute_head_with_micro_batches_is_recorded():
+    """Every pass of an update is recorded, the accumulating ones of the recomputing head too: a recording that had to be given up
+    would have left the reason in the model's last error."""
+    rng = np.random.default_rng(5)
+    m = _model(rng, head_mode="recompute")
+    parts = [_batch(rng, 4, 48) for _ in range(3)]
+    first = None
+    for _ in range(4):
+        m.set_micro_batches(3)
+        for b in parts:
+            r = _result(m, b)
+        first = first or r
+        for x, y in zip(first, r):
+            assert np.array_equal(x, y)
+        assert m.L.il_last_error(m._h) == b""
