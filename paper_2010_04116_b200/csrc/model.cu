@@ -1575,19 +1575,20 @@ extern "C" il_status il_sync(il_model* m) {
     IL_CUDA(m, cudaSetDevice(m->dev[k]));
     IL_CUDA(m, cudaStreamSynchronize(m->streams[k]));
   }
-  // error word and per-component update counters of every distinct buffer
+  // error word and update counters, of the components and of their heads' matrices, of every distinct buffer
   unsigned first = 0;
   int applied_min = m->adamw_issued, applied_max = 0;
-  unsigned words[1 + 64];                 // K <= 64 (il_create)
+  unsigned words[1 + 2 * 64];             // K <= 64 (il_create)
   const bool shared = m->err_word[m->K - 1] == m->err_word[0];
   for (int k = 0; k < m->K; ++k) {
     if (shared && k > 0) break;
-    IL_TRY(copy_sync(m, k, words, m->err_word[k], 4 * (size_t)(1 + m->K), cudaMemcpyDeviceToHost));
+    IL_TRY(copy_sync(m, k, words, m->err_word[k], 4 * (size_t)(1 + 2 * m->K), cudaMemcpyDeviceToHost));
     if (words[0] && !first) first = words[0];
-    for (int j = shared ? 0 : k; j <= (shared ? m->K - 1 : k); ++j) {
-      applied_min = std::min(applied_min, (int)words[1 + j]);
-      applied_max = std::max(applied_max, (int)words[1 + j]);
-    }
+    for (int j = shared ? 0 : k; j <= (shared ? m->K - 1 : k); ++j)
+      for (int c : {(int)words[1 + j], (int)words[1 + m->K + j]}) {
+        applied_min = std::min(applied_min, c);
+        applied_max = std::max(applied_max, c);
+      }
     IL_CUDA(m, cudaMemsetAsync(m->err_word[k], 0, 4 * (size_t)(1 + 2 * m->K), m->streams[k]));
     IL_CUDA(m, cudaStreamSynchronize(m->streams[k]));
   }
@@ -1595,9 +1596,10 @@ extern "C" il_status il_sync(il_model* m) {
   m->adamw_issued = 0;
   if (first) {
     // Updates enqueued after the failure were skipped on the device: the step counter goes back to the number of
-    // updates that were applied.  A component whose update ran before another component raised the error keeps it.
+    // updates that were applied.  What was updated before something else raised the error, a component or a head's
+    // vocabulary matrix, keeps it.
     m->step -= (issued - applied_max);
-    const char* partial = applied_min != applied_max ? "; some components applied an update that others skipped" : "";
+    const char* partial = applied_min != applied_max ? "; some components or heads' matrices applied an update that others skipped" : "";
     if (first == DEV_LOGIT_RANGE) {
       // Only the stored-exp(logit) head has this limit.  From here on the model recomputes the logits in the head
       // backward instead (the stored matrix's memory becomes the chunk buffer); the caller repeats the step.

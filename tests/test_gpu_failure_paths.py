@@ -85,6 +85,33 @@ def test_update_is_skipped_while_the_error_word_is_set():
         m.close()
 
 
+def test_a_head_update_before_the_error_is_reported_as_applied():
+    """The vocabulary matrix's update follows its head's backward; an error raised after that keeps the rest of the component
+    from its own.  il_sync says so and the step counter stays: repeating the step would update the matrix twice."""
+    m = Model(1, 1, 64, 2, 128, 300, 1, 2, 16)
+    try:
+        rng = np.random.default_rng(2)
+        for nm in m.names:
+            m.set_param(nm, (rng.standard_normal(m.shapes[nm]) * 0.05 + nm.endswith(".g")).astype(np.float32))
+        batch = [rng.integers(0, 300, size=(2, 16)).astype(np.int32) for _ in range(2)]
+        m.train_step(*batch, adamw=HP)                   # (a kernel's first launch may wait for what is running)
+        m.sync()
+        before = {nm: m.get_param(nm) for nm in ("head0.w", "c0.l0.mlp.w1")}
+        m.train_step(*batch)
+        torch.cuda.synchronize()
+        il.op_wait_probe(m.error_word(0), 500000, m.streams[0].cuda_stream)      # the error, half a second from now
+        m.adamw_step(**HP)
+        with pytest.raises(ILError) as e:
+            m.sync()
+        assert e.value.status == 5
+        assert not np.array_equal(m.get_param("head0.w"), before["head0.w"])
+        assert np.array_equal(m.get_param("c0.l0.mlp.w1"), before["c0.l0.mlp.w1"])
+        assert "1 of 1 optimiser updates" in str(e.value) and "others skipped" in str(e.value)
+        assert m.get_opt_state("head0.w")[2] == 2
+    finally:
+        m.close()
+
+
 def test_recompute_head_has_no_logit_range_limit():
     w, m, P, tok, tgt = _small(n=1, head_mode="recompute")
     try:
