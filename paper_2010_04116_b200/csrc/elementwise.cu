@@ -105,7 +105,8 @@ __global__ void __launch_bounds__(1024) embed_sort_kernel(const int* __restrict_
 size_t embed_sort_words(size_t ntok) { return (ntok + SORT_CHUNK - 1) / SORT_CHUNK * SORT_STRIDE; }
 
 cudaError_t embed_sort(const int* tok, unsigned* keys, int ntok, int V, cudaStream_t s) {
-  if (V > (1 << (32 - SORT_POS_BITS)) - 1) return cudaErrorInvalidValue;
+  static_assert(EMBED_SORT_MAX_V == (1 << (32 - SORT_POS_BITS)) - 1, "a key is token << SORT_POS_BITS | position, none of them ~0");
+  if (V > EMBED_SORT_MAX_V) return cudaErrorInvalidValue;
   launch_dep(embed_sort_kernel, dim3(ceil_div(ntok, SORT_CHUNK)), dim3(1024), 0, s, tok, keys, ntok, V);
   return cudaGetLastError();
 }

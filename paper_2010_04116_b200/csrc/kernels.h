@@ -11,7 +11,8 @@ namespace il {
 cudaError_t embed_fwd(const int* tok, const float* wte, const float* wpe, float* x, int ntok, int T, int d, int V,
                       cudaStream_t s);
 // keys [embed_sort_words(ntok)] = the batch's (token, position) pairs in sorted order and the runs of equal tokens, for
-// embed_bwd.  V < 2^19.
+// embed_bwd.
+constexpr int EMBED_SORT_MAX_V = (1 << 19) - 1;
 size_t embed_sort_words(size_t ntok);
 cudaError_t embed_sort(const int* tok, unsigned* keys, int ntok, int V, cudaStream_t s);
 // dwte[t,:] = (accumulate ? dwte[t,:] : 0) + sum over the positions i with tok[i] = t of dx[i,:], summed in position

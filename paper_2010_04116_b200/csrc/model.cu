@@ -930,6 +930,8 @@ extern "C" il_status il_set_batch(il_model* m, const int* tokens, const int* tar
   if (!tokens || !targets) return fail(m, IL_ERR_INVALID_ARG, "NULL tokens/targets");
   if (B < 1 || T < 1 || B > m->max_batch || T > m->max_seq || (size_t)B * T > (size_t)m->ntok_max)
     return fail(m, IL_ERR_INVALID_ARG, "batch %dx%d exceeds max_batch=%d, max_seq=%d", B, T, m->max_batch, m->max_seq);
+  // (here, before any work, and not in the middle of the backward that needs the sort)
+  if (m->V > EMBED_SORT_MAX_V) return fail(m, IL_ERR_CUDA, "vocabulary of %d ids: the token sort takes up to %d", m->V, EMBED_SORT_MAX_V);
   IL_CUDA(m, cudaSetDevice(m->dev[0]));
   // every stream's previous work must be finished before buffers of the last step are overwritten
   IL_TRY(join_all(m));

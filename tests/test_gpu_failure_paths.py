@@ -112,6 +112,19 @@ def test_a_head_update_before_the_error_is_reported_as_applied():
         m.close()
 
 
+def test_vocabulary_beyond_the_sort_keys_is_refused_with_the_batch():
+    m = Model(1, 1, 32, 1, 64, 2 ** 19, 1, 1, 8)
+    try:
+        tok = np.zeros((1, 8), dtype=np.int32)
+        with pytest.raises(ILError):
+            m.set_batch(tok, tok)
+        with pytest.raises(ILError) as e:
+            m.forward_component(0)
+        assert e.value.status == 2
+    finally:
+        m.close()
+
+
 def test_recompute_head_has_no_logit_range_limit():
     w, m, P, tok, tgt = _small(n=1, head_mode="recompute")
     try:
