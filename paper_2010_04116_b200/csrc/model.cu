@@ -113,7 +113,9 @@ struct il_model {
   // Parameter gradients of a small backward pass run on a branch of the component's stream (BackwardBranch).
   std::vector<cudaStream_t> branch;
   std::vector<cudaEvent_t> ev_fork, ev_branch[3];
-  cudaEvent_t ev_batch, ev_sort;      // the batch is on the device; its token keys are sorted
+  cudaEvent_t ev_batch;               // the batch is on the device
+  cudaEvent_t ev_unsorted, ev_sort;   // stream 0 has come to the backward; the batch's token keys are sorted
+  bool sort_pending;                  // a sort has been enqueued that stream 0 has not been made to wait for
   // parameters
   std::vector<TensorRec> tensors;
   std::vector<LayerOff> layer_off;   // K*Lc main layers, then K*Lh head layers (head k's at K*Lc + k*Lh)
@@ -501,6 +503,7 @@ extern "C" il_status il_create(int K, int Lc, int d, int H, int F, int V, int n,
   m->prof = 0; m->batch_set = false; m->bwd_done = false;
   m->B = m->T = m->ntok = 0;
   m->ev_batch = nullptr;
+  m->ev_unsorted = m->ev_sort = nullptr; m->sort_pending = false;
   *out = m;   // returned even on failure below so that il_last_error/il_destroy work
 
   auto bail = [&](il_status s) { return s; };
@@ -648,6 +651,7 @@ extern "C" il_status il_create(int K, int Lc, int d, int H, int F, int V, int n,
   }
   IL_CUDA(m, cudaSetDevice(m->dev[0]));
   IL_CUDA(m, cudaEventCreateWithFlags(&m->ev_batch, cudaEventDisableTiming));
+  IL_CUDA(m, cudaEventCreateWithFlags(&m->ev_unsorted, cudaEventDisableTiming));
   IL_CUDA(m, cudaEventCreateWithFlags(&m->ev_sort, cudaEventDisableTiming));
 
   // ---- parameter, gradient and optimiser storage
@@ -799,6 +803,7 @@ extern "C" il_status il_destroy(il_model* m) {
   for (auto st : m->side) cudaStreamDestroy(st);
   for (auto st : m->branch) cudaStreamDestroy(st);
   if (m->ev_batch) cudaEventDestroy(m->ev_batch);
+  if (m->ev_unsorted) cudaEventDestroy(m->ev_unsorted);
   if (m->ev_sort) cudaEventDestroy(m->ev_sort);
   for (auto e : m->prof_pool) cudaEventDestroy(e);
   for (auto& r : m->prof_recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
@@ -937,7 +942,13 @@ extern "C" il_status il_set_batch(il_model* m, const int* tokens, const int* tar
   IL_TRY(join_all(m));
   cudaStream_t s0 = m->streams[0];
   const size_t bytes = (size_t)B * T * sizeof(int);
-  IL_CUDA(m, cudaStreamWaitEvent(s0, m->ev_sort, 0));     // the last batch's ids have been read by the sort
+  // The last batch's ids have been read by the sort.  Stream 0 knows unless a backward was given up half way.  (A caller may be
+  // capturing the streams, and a capture must not wait for events from outside of it: every event waited for in a step
+  // has been recorded in that step.)
+  if (m->sort_pending) {
+    IL_CUDA(m, cudaStreamWaitEvent(s0, m->ev_sort, 0));
+    m->sort_pending = false;
+  }
   const cudaMemcpyKind kind = on_device ? cudaMemcpyDefault : cudaMemcpyHostToDevice;
   IL_CUDA(m, cudaEventRecord(m->ev_batch, s0));
   for (int k = 0; k < m->K; ++k) {
@@ -972,6 +983,11 @@ template <class F>
 il_status run_segment(il_model* m, int kind, int k, const int (&key)[6], F&& body) {
   cudaStream_t st = m->streams[k];
   if (m->prof) return body();                    // (timing of single GEMMs needs their events)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return body();                               // the caller is capturing the stream: the launches go into that graph
+  }
   Segment* s = nullptr;
   for (Segment& c : m->segments[k])
     if (c.kind == kind && memcmp(c.key, key, sizeof key) == 0) { s = &c; break; }
@@ -996,8 +1012,7 @@ il_status run_segment(il_model* m, int kind, int k, const int (&key)[6], F&& bod
   }
   s->stamp = ++m->segment_clock;
   if (!s->exec) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (s->uses < 1 || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    if (s->uses < 1) {
       if (s->uses >= 0) s->uses++;
       return body();
     }
@@ -1333,7 +1348,10 @@ il_status head_backward(il_model* m, int k, bool acc, float scale) {
 template <class G>
 il_status component_backward(il_model* m, int k, int s, bool acc, G&& gather) {
   cudaStream_t st = m->streams[k];
-  if (k == 0) IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_sort, 0));
+  if (k == 0) {
+    IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_sort, 0));
+    m->sort_pending = false;
+  }
   const int key[6] = {m->B, m->T, s, acc ? 1 : 0, m->n, m->rule};
   return run_segment(m, SEG_COMPONENT_BACKWARD, k, key, [&]() -> il_status {
     IL_TRY(gather());
@@ -1384,6 +1402,8 @@ extern "C" il_status il_backward_nwise(il_model* m) {
   const bool acc = m->micro > 1 && m->micro_done > 0;
   const float gscale = 1.0f / (float)m->micro;
 
+  IL_CUDA(m, cudaSetDevice(m->dev[0]));
+  IL_CUDA(m, cudaEventRecord(m->ev_unsorted, m->streams[0]));
   // every head's own backward is independent of the others: enqueue all of them first
   for (int k = 0; k < K; ++k) {
     cudaStream_t st = m->streams[k];
@@ -1395,12 +1415,13 @@ extern "C" il_status il_backward_nwise(il_model* m) {
     }
     IL_CUDA(m, cudaEventRecord(m->ev_head[k], st));      // head k's parameter gradients are final from here on
   }
-  // (token, position) keys in sorted order for the embedding backward: made on component 0's side stream beside all that comes
-  // before it (44 us for 8192 positions; a forward pass without a backward does not need them)
+  // (token, position) keys in sorted order for the embedding backward: made on component 0's side stream beside the backward
+  // passes that come before it (44 us for 8192 positions; a forward pass without a backward does not need them)
   IL_CUDA(m, cudaSetDevice(m->dev[0]));
-  IL_CUDA(m, cudaStreamWaitEvent(m->side[0], m->ev_batch, 0));
+  IL_CUDA(m, cudaStreamWaitEvent(m->side[0], m->ev_unsorted, 0));
   IL_K(m, embed_sort(m->tokens[0], m->sort_keys[0], N, m->V, m->side[0]));
   IL_CUDA(m, cudaEventRecord(m->ev_sort, m->side[0]));
+  m->sort_pending = true;
   if (m->rule == IL_RULE_SUM) {
     // components from the top down; component k needs the pass-down of component k+1 when any stream crosses
     std::vector<int> above;   // termination levels of the streams of component k+1

@@ -77,3 +77,44 @@ def test_recompute_head_with_micro_batches_is_recorded():
         for x, y in zip(first, r):
             assert np.array_equal(x, y)
         assert m.L.il_last_error(m._h) == b""
+
+
+@pytest.mark.parametrize("kw", [{"K": 2}, {"K": 1, "n": 1}, {"K": 3, "Lh": 1, "head_mode": "recompute"}])
+@pytest.mark.parametrize("with_batch", [True, False])
+def test_a_caller_captures_a_step(kw, with_batch):
+    """A step whose streams the caller is capturing goes into the caller's graph, after steps outside of it and before others, with
+    the batch's copy or without it (then the graph runs on whatever batch is set before it)."""
+    rng = np.random.default_rng(6)
+    m = _model(rng, **kw)
+    batches = [tuple(torch.tensor(x, device="cuda") for x in _batch(rng, 4, 48)) for _ in range(2)]
+    ref = [_result(m, b) for b in batches]
+    weights = [name for name in m.names if len(m.shapes[name]) == 2]
+    graph = torch.cuda.CUDAGraph()
+    if not with_batch:
+        m.set_batch(*batches[0])
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=m.streams[0]):
+        for s in m.streams[1:]:
+            s.wait_stream(m.streams[0])
+        if with_batch:
+            m.set_batch(*batches[0])
+        for k in range(m.K):
+            m.forward_component(k)
+            m.aux_head_loss(k)
+        m.backward_nwise()
+        for s in m.streams[1:]:
+            m.streams[0].wait_stream(s)
+    for i in [0] if with_batch else [0, 1, 0]:
+        if not with_batch:
+            _result(m, batches[i])                        # (as a step; what follows runs on the same ids)
+        list(m._blocks.values())[1].fill_(77)             # the gradients
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        for x, name in zip(ref[i][1:], weights):
+            assert np.array_equal(x, m.get_grad(name)), name
+    del graph
+    for i in [0, 1, 1, 0]:
+        for x, y in zip(ref[i], _result(m, batches[i])):
+            assert np.array_equal(x, y)
+    assert m.L.il_last_error(m._h) == b""
