@@ -975,10 +975,43 @@ extern "C" il_status il_set_batch(il_model* m, const int* tokens, const int* tar
 
 namespace {
 
-// Enqueue `body` (work on component k's stream only: kernels, memsets and copies between the model's own buffers, no
-// events) directly the first time, and as a recorded graph from the second time on.  A tiny step is ~100 kernels of
-// 2-4 us; enqueued one by one each costs the host about 4 us (tensor maps, launch attributes), a graph of them 5-10 us
-// in all.  Nothing in a recording refers to a caller's buffer: the batch is copied into the model's own memory first.
+// Recording of what is enqueued on component k's stream.  It is made on the component's side stream, which stands in for
+// streams[k] meanwhile and which nobody outside the model can reach: a caller's stream that is being captured would take in whatever
+// else is put on it (another thread's kernels, another model's steps on a shared stream), and could make calls on the legacy
+// stream fail elsewhere in the process.
+struct Recording {
+  il_model* m;
+  int k;
+  cudaStream_t own;
+  bool open;
+  Recording(il_model* m_, int k_) : m(m_), k(k_), own(m_->streams[k_]), open(false) {}
+  bool begin() {
+    if (cudaStreamBeginCapture(m->side[k], cudaStreamCaptureModeThreadLocal) != cudaSuccess) return false;
+    open = true;
+    m->streams[k] = m->side[k];
+    return true;
+  }
+  // The recording, ready to be launched; NULL if it is not wanted or could not be made.
+  cudaGraphExec_t end(bool wanted) {
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    if (open) {
+      open = false;
+      m->streams[k] = own;
+      if (cudaStreamEndCapture(m->side[k], &g) != cudaSuccess || !wanted || cudaGraphInstantiate(&exec, g, 0) != cudaSuccess) exec = nullptr;
+      if (g) cudaGraphDestroy(g);
+    }
+    if (!exec) cudaGetLastError();
+    return exec;
+  }
+  ~Recording() { end(false); }           // (an exception on the way)
+};
+
+// Enqueue `body` (kernels, memsets and copies between the model's own buffers, on component k's stream, taken from streams[k] when it
+// runs, and on branches that fork from and join it) directly the first time, and as a recorded graph from the second time
+// on.  A tiny step is ~100 kernels of 2-4 us; enqueued one by one each costs the host about 4 us (tensor maps, launch attributes),
+// a graph of them 5-10 us in all.  Nothing in a recording refers to a caller's buffer: the batch is copied into the model's own
+// memory first.
 template <class F>
 il_status run_segment(il_model* m, int kind, int k, const int (&key)[6], F&& body) {
   cudaStream_t st = m->streams[k];
@@ -1016,26 +1049,16 @@ il_status run_segment(il_model* m, int kind, int k, const int (&key)[6], F&& bod
       if (s->uses >= 0) s->uses++;
       return body();
     }
+    Recording rec(m, k);
     const long long l0 = m->launches;
-    if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-      cudaGetLastError();
-      s->uses = -1;
-      return body();
-    }
-    const il_status rs = body();
-    cudaGraph_t g = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(st, &g);
+    const bool whole = rec.begin() && body() == IL_OK;
+    s->exec = rec.end(whole);
     s->launches = m->launches - l0;
     m->launches = l0;
-    cudaGraphExec_t exec = nullptr;
-    if (rs != IL_OK || e != cudaSuccess || !g || cudaGraphInstantiate(&exec, g, 0) != cudaSuccess) {
-      cudaGetLastError();
-      if (g) cudaGraphDestroy(g);
+    if (!s->exec) {
       s->uses = -1;
       return body();
     }
-    cudaGraphDestroy(g);
-    s->exec = exec;
   }
   IL_CUDA(m, cudaGraphLaunch(s->exec, st));
   m->launches += s->launches;
@@ -1105,7 +1128,7 @@ extern "C" il_status il_forward_component(il_model* m, int k) {
   {
     const int key[6] = {m->B, m->T, 0, 0, 0, 0};
     IL_TRY(run_segment(m, SEG_FORWARD, k, key, [&]() -> il_status {
-      if (k == 0) IL_K(m, embed_fwd(m->tokens[k], m->P[k] + m->off_wte, m->P[k] + m->off_wpe, m->a[0], N, m->T, d, m->V, st));
+      if (k == 0) IL_K(m, embed_fwd(m->tokens[k], m->P[k] + m->off_wte, m->P[k] + m->off_wpe, m->a[0], N, m->T, d, m->V, m->streams[k]));
       return layers_forward(m, k, (size_t)k * m->Lc, m->Lc, comp_input(m, k));
     }));
   }
@@ -1126,6 +1149,7 @@ extern "C" il_status il_aux_head_loss(il_model* m, int k, float* loss_host) {
   if (!m->loss_done[k]) {
     const int key[6] = {m->B, m->T, m->head_mode, 0, 0, 0};
     IL_TRY(run_segment(m, SEG_HEAD_LOSS, k, key, [&]() -> il_status {
+    cudaStream_t st = m->streams[k];
     const int N = m->ntok, d = m->d, V = m->V;
     const HeadOff& o = m->head_off[k];
     HeadScratch& h = m->hs[k];
@@ -1343,18 +1367,18 @@ il_status head_backward(il_model* m, int k, bool acc, float scale) {
   return IL_OK;
 }
 
-// Backward of component k for s stacked gradient streams, which `gather` puts in place (kernels on stream k that depend on
+// Backward of component k for s stacked gradient streams, which `gather` puts in place (kernels on the stream it is given that depend on
 // nothing but the rule and the window), down to the embedding's gradients below component 0.
 template <class G>
 il_status component_backward(il_model* m, int k, int s, bool acc, G&& gather) {
-  cudaStream_t st = m->streams[k];
   if (k == 0) {
-    IL_CUDA(m, cudaStreamWaitEvent(st, m->ev_sort, 0));
+    IL_CUDA(m, cudaStreamWaitEvent(m->streams[k], m->ev_sort, 0));
     m->sort_pending = false;
   }
   const int key[6] = {m->B, m->T, s, acc ? 1 : 0, m->n, m->rule};
   return run_segment(m, SEG_COMPONENT_BACKWARD, k, key, [&]() -> il_status {
-    IL_TRY(gather());
+    cudaStream_t st = m->streams[k];
+    IL_TRY(gather(st));
     IL_TRY(layers_backward(m, k, s, (size_t)k * m->Lc, m->Lc, comp_input(m, k), acc));
     if (k == 0) {
       IL_K(m, embed_bwd(m->tokens[k], m->sort_keys[0], m->cs[0].dx, m->G[k] + m->off_wte, m->G[k] + m->off_wpe, m->ntok, m->T, m->d,
@@ -1446,9 +1470,9 @@ extern "C" il_status il_backward_nwise(il_model* m) {
       }
       {
         Range r2("component backward %d", k);
-        IL_TRY(component_backward(m, k, s, acc, [&]() -> il_status {
+        IL_TRY(component_backward(m, k, s, acc, [&](cudaStream_t on) -> il_status {
           for (int j = 0; j < s; ++j)
-            IL_K(m, add_convert(m->hs[k].ghead, pass[j], m->cs[k].dx + (size_t)j * slice, m->cs[k].dxb + (size_t)j * slice, slice, st));
+            IL_K(m, add_convert(m->hs[k].ghead, pass[j], m->cs[k].dx + (size_t)j * slice, m->cs[k].dxb + (size_t)j * slice, slice, on));
           return IL_OK;
         }));
       }
@@ -1506,13 +1530,13 @@ extern "C" il_status il_backward_nwise(il_model* m) {
       if (fetch_err != cudaSuccess) return fail(m, IL_ERR_CUDA, "cudaMemcpyPeerAsync: %s", cudaGetErrorString(fetch_err));
       {
         Range r2("component backward %d", k);
-        IL_TRY(component_backward(m, k, used, acc, [&]() -> il_status {
+        IL_TRY(component_backward(m, k, used, acc, [&](cudaStream_t on) -> il_status {
           for (int c0 = 0; c0 < cnt; c0 += 4) {
             const int c = cnt - c0 < 4 ? cnt - c0 : 4;
-            IL_K(m, lincomb_convert(xs + c0, ws + c0, c, c0 > 0, m->cs[k].dx, c0 + 4 >= cnt ? m->cs[k].dxb : nullptr, slice, st));
+            IL_K(m, lincomb_convert(xs + c0, ws + c0, c, c0 > 0, m->cs[k].dx, c0 + 4 >= cnt ? m->cs[k].dxb : nullptr, slice, on));
           }
           for (int j = 1; j < used; ++j)
-            IL_K(m, add_convert(relay[j], nullptr, m->cs[k].dx + (size_t)j * slice, m->cs[k].dxb + (size_t)j * slice, slice, st));
+            IL_K(m, add_convert(relay[j], nullptr, m->cs[k].dx + (size_t)j * slice, m->cs[k].dxb + (size_t)j * slice, slice, on));
           return IL_OK;
         }));
       }

@@ -1,4 +1,6 @@
 """The parts of a step that are replayed as recorded graphs from their second use on give the bits of the first use."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -118,3 +120,36 @@ def test_a_caller_captures_a_step(kw, with_batch):
         for x, y in zip(ref[i], _result(m, batches[i])):
             assert np.array_equal(x, y)
     assert m.L.il_last_error(m._h) == b""
+
+
+def test_other_work_on_the_model_s_streams_is_not_recorded():
+    """Another thread's kernels on a stream that the model works on (two models may share one of torch's streams) run once each."""
+    rng = np.random.default_rng(7)
+    m = _model(rng)
+    counters = torch.zeros(len(m.streams), device="cuda")
+    torch.cuda.synchronize()
+    issued, stop, failed = [0] * len(m.streams), threading.Event(), []
+
+    def other():
+        try:
+            while not stop.is_set():
+                for i, s in enumerate(m.streams):
+                    with torch.cuda.stream(s):
+                        counters[i].add_(1)
+                    issued[i] += 1
+        except Exception as e:
+            failed.append(e)
+    t = threading.Thread(target=other)
+    t.start()
+    try:
+        for B in range(1, 5):
+            for T in range(1, 13):
+                b = _batch(rng, B, T)
+                for _ in range(3):
+                    _result(m, b)
+    finally:
+        stop.set()
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed
+    assert counters.tolist() == issued
