@@ -61,7 +61,7 @@ struct HeadScratch {
 };
 
 // A stretch of one component stream's work that depends on nothing but the model's own buffers and a few integers (the
-// key), recorded as a CUDA graph when it is asked for a second time and replayed from then on.
+// key), recorded as a CUDA graph when it is asked for a second time, if there is room, and replayed from then on.
 struct Segment {
   int kind, k;
   int key[6];
@@ -70,7 +70,12 @@ struct Segment {
   cudaGraphExec_t exec;
 };
 enum { SEG_FORWARD, SEG_HEAD_LOSS, SEG_HEAD_BACKWARD, SEG_COMPONENT_BACKWARD };
-constexpr size_t SEGMENTS_PER_STREAM = 16;     // four kinds, a few batch shapes each; the least recently used one goes
+// A component keeps up to 16 recordings: four kinds (six with micro-batches) for a few batch shapes.  One gives way only after
+// 1024 calls on its stream without a use, 256 steps; until then what finds no room is enqueued directly.  (When the least recently
+// used one gave way at once, more shapes than fit were recorded and dropped in turn: K = 2 x 2 layers of d 128, 8 lengths in
+// random order 810 us a step, enqueued directly 380, all recorded 330.)  Keys are remembered beyond the recordings.
+constexpr size_t SEGMENTS_RECORDED = 16, SEGMENTS_KNOWN = 256;
+constexpr long long SEGMENT_IDLE = 1024;
 
 struct ProfRec { cudaEvent_t a, b; double flops; };
 
@@ -163,7 +168,7 @@ struct il_model {
   int prof;                           // 0 off, 1 events around each GEMM, 2 the same with the GEMM alone on the GPU
   std::vector<ProfRec> prof_recs;
   std::vector<std::vector<Segment>> segments;   // per component
-  long long segment_clock;
+  std::vector<long long> segment_clock;         // calls of run_segment so far
   std::vector<cudaEvent_t> prof_pool;
   std::string err;
 };
@@ -499,7 +504,7 @@ extern "C" il_status il_create(int K, int Lc, int d, int H, int F, int V, int n,
   m->max_batch = opt->max_batch; m->max_seq = opt->max_seq;
   m->ntok_max = opt->max_batch * opt->max_seq;
   m->ln_eps = opt->ln_eps > 0 ? opt->ln_eps : 1e-5f;
-  m->rule = IL_RULE_SUM; m->step = 0; m->adamw_issued = 0; m->segment_clock = 0; m->segments.resize((size_t)K); m->bytes = 0; m->launches = 0; m->s_cap = 0;
+  m->rule = IL_RULE_SUM; m->step = 0; m->adamw_issued = 0; m->segment_clock.assign((size_t)K, 0); m->segments.resize((size_t)K); m->bytes = 0; m->launches = 0; m->s_cap = 0;
   m->prof = 0; m->batch_set = false; m->bwd_done = false;
   m->B = m->T = m->ntok = 0;
   m->ev_batch = nullptr;
@@ -1021,21 +1026,19 @@ il_status run_segment(il_model* m, int kind, int k, const int (&key)[6], F&& bod
     cudaGetLastError();
     return body();                               // the caller is capturing the stream: the launches go into that graph
   }
+  std::vector<Segment>& v = m->segments[k];
   Segment* s = nullptr;
-  for (Segment& c : m->segments[k])
+  for (Segment& c : v)
     if (c.kind == kind && memcmp(c.key, key, sizeof key) == 0) { s = &c; break; }
+  // the least recently used of the recordings, or of the keys that have none
+  auto oldest = [&](bool recorded) {
+    size_t old = v.size();
+    for (size_t i = 0; i < v.size(); ++i)
+      if ((v[i].exec != nullptr) == recorded && (old == v.size() || v[i].stamp < v[old].stamp)) old = i;
+    return old;
+  };
   if (!s) {
-    std::vector<Segment>& v = m->segments[k];
-    if (v.size() >= SEGMENTS_PER_STREAM) {
-      size_t old = 0;
-      for (size_t i = 1; i < v.size(); ++i)
-        if (v[i].stamp < v[old].stamp) old = i;
-      if (v[old].exec) {
-        IL_CUDA(m, cudaStreamSynchronize(st));                 // its last launch may still be running
-        cudaGraphExecDestroy(v[old].exec);
-      }
-      v.erase(v.begin() + (long)old);
-    }
+    if (v.size() >= SEGMENTS_KNOWN) v.erase(v.begin() + (long)oldest(false));
     Segment n;
     memset(&n, 0, sizeof n);
     n.kind = kind; n.k = k;
@@ -1043,11 +1046,19 @@ il_status run_segment(il_model* m, int kind, int k, const int (&key)[6], F&& bod
     v.push_back(n);
     s = &v.back();
   }
-  s->stamp = ++m->segment_clock;
+  const long long now = ++m->segment_clock[k];
+  s->stamp = now;
   if (!s->exec) {
     if (s->uses < 1) {
-      if (s->uses >= 0) s->uses++;
+      if (s->uses == 0) s->uses = 1;
       return body();
+    }
+    if (std::count_if(v.begin(), v.end(), [](const Segment& c) { return c.exec != nullptr; }) >= (long)SEGMENTS_RECORDED) {
+      Segment& old = v[oldest(true)];
+      if (now - old.stamp < SEGMENT_IDLE) return body();
+      IL_CUDA(m, cudaStreamSynchronize(st));                   // its last launch may still be running
+      cudaGraphExecDestroy(old.exec);
+      old.exec = nullptr;
     }
     Recording rec(m, k);
     const long long l0 = m->launches;

@@ -153,3 +153,40 @@ def test_other_work_on_the_model_s_streams_is_not_recorded():
     torch.cuda.synchronize()
     assert not failed
     assert counters.tolist() == issued
+
+
+def test_more_shapes_than_recordings_are_not_recorded_over_and_over():
+    """Batch shapes in random order, more of them than a component keeps recordings for: those it has stay in use, the others are
+    enqueued directly, and nothing waits for the stream in the middle of a step."""
+    rng = np.random.default_rng(8)
+    m = _model(rng)
+    batches = [_batch(rng, 4, T) for T in range(6, 48, 4)]
+    for i in rng.permutation(np.arange(8 * len(batches)) % len(batches)):
+        m.train_step(*batches[i])
+        m.sync()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU, torch.profiler.ProfilerActivity.CUDA]) as prof:
+        for i in rng.permutation(np.arange(4 * len(batches)) % len(batches)):
+            m.train_step(*batches[i])
+    calls = {e.key: e.count for e in prof.key_averages()}
+    assert sum(n for name, n in calls.items() if "GraphLaunch" in name) > 0, calls
+    assert not [name for name in calls if "GraphInstantiate" in name or "StreamSynchronize" in name], calls
+
+
+def test_recordings_follow_a_program_to_other_shapes():
+    """Recordings that nobody has used for 1024 calls on their stream make room."""
+    rng = np.random.default_rng(9)
+    m = _model(rng)
+    for T in range(6, 48, 4):
+        b = _batch(rng, 4, T)
+        for _ in range(3):
+            m.train_step(*b)
+    b = _batch(rng, 4, 48)
+    first = _result(m, b)
+    for i in range(270):
+        m.train_step(*b)
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU, torch.profiler.ProfilerActivity.CUDA]) as prof:
+        m.train_step(*b)
+    calls = {e.key: e.count for e in prof.key_averages()}
+    assert sum(n for name, n in calls.items() if "GraphLaunch" in name) == 4 * m.K, calls
+    for x, y in zip(first, _result(m, b)):
+        assert np.array_equal(x, y)
