@@ -57,8 +57,9 @@ typedef struct {
   int tile_blocks; /* output tile: 1 = 256 x 256, 2 = 256 x 512 (fewer operand bytes per product, epilogue less
                       hidden); negative: one CTA per tile, -S (128 x 128) or -(64 + S) (128 x 64) with the
                       contraction split over a cluster of S = 1, 2, 4 or 8 CTAs and added in rank order
-                      (epilogues 0-4 in the layouts of the training step); 0 = chosen from the shape.  The
-                      choice changes nothing but the order of the fp32 sums */
+                      (epilogues 0-4 in the layouts of the training step); 0, and whatever names no form of the
+                      product's epilogue and layout = chosen from the shape.  The choice changes nothing but the
+                      order of the fp32 sums */
   const float* rowscale; /* epilogue 4 */
   int store_exp;         /* epilogue 5 */
 } il_gemm_desc;

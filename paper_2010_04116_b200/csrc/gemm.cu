@@ -732,11 +732,12 @@ cudaError_t gemm_launch(const GemmArgs& a, unsigned* err_word, int num_sms, cuda
     plan.tn = 0;
     plan.nt = a.tile_blocks == 1 || a.tile_blocks == 2 ? a.tile_blocks : (a.N > BN && a.K >= 2048) ? 2 : 1;
     if (a.N <= BN) plan.nt = 1;
-  } else if (a.tile_blocks < 0) {
-    plan.tn = -a.tile_blocks & 64 ? 64 : 128;
-    plan.split = -a.tile_blocks & 15;
-    if (plan.split != 1 && plan.split != 2 && plan.split != 4 && plan.split != 8) return cudaErrorInvalidValue;
-    if (!gemm_small_supported(a.A.mn_major, a.B.mn_major, a.epilogue)) return cudaErrorInvalidValue;
+  } else if (a.tile_blocks < 0) {                // the single-CTA kernel where it has the form (otherwise as the shape has it)
+    const int tn = a.tile_blocks <= -64 ? 64 : 128, split = -a.tile_blocks - (tn == 64 ? 64 : 0);
+    if ((split == 1 || split == 2 || split == 4 || split == 8) && gemm_small_supported(a.A.mn_major, a.B.mn_major, a.epilogue)) {
+      plan.tn = tn;
+      plan.split = split;
+    }
   }
   const int nt = plan.nt;
   KernelFn kern = pick_kernel(a.A.mn_major, a.B.mn_major, a.epilogue, nt);

@@ -55,7 +55,7 @@ struct GemmArgs {
   int store_exp;      // EPI_LSE with C: store exp(acc) instead of acc
   int tile_blocks;    // 256-column blocks per output tile of a CTA pair: 1 (256 x 256), 2 (256 x 512); negative: tiles of one
                       // CTA, -S (128 x 128) or -(64 + S) (128 x 64) with the contraction split over a cluster of S = 1,
-                      // 2, 4, 8 CTAs; 0 = chosen from the shape
+                      // 2, 4, 8 CTAs; 0, and what the single-CTA kernel does not have = chosen from the shape
   int concurrency;    // streams that run work like this at the same time (0 = 1): weighs latency against SM time
 };
 

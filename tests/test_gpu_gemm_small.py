@@ -85,3 +85,26 @@ def test_cluster_split_gemm(M, N, K, layout, epi, tile):
         assert rel(act[:, :N], act_ref) < 3e-3
     if cs is not None:
         assert rel(cs[:N], ref[:(M + 1) // 2].sum(0)) < 4 * tol32
+
+
+@pytest.mark.parametrize("tile", [-1, -8, -66, -3, -200, 7])
+def test_tile_the_epilogue_does_not_have_is_chosen_from_the_shape(tile):
+    """A tile_blocks that names no form of the product's epilogue and layout leaves the choice to the shape."""
+    M, N, K = 130, 300, 72
+    A, B, ref, g = _case(M, N, K, (0, 0), 5, 9)
+    targets = torch.randint(0, N, (M,), device=DEV, generator=g).to(torch.int32)
+    err = torch.zeros(1, dtype=torch.int32, device=DEV)
+    res = []
+    for t in (0, tile):
+        part = [torch.zeros(M, 3, device=DEV) for _ in range(2)]
+        tgt = torch.zeros(M, device=DEV)
+        il.op_gemm(M, N, K, A, A.shape[1], 0, B, B.shape[1], 0, 5, err, targets=targets, part_max=part[0], part_sum=part[1], part_ld=3,
+                   tgt_logit=tgt, tile_blocks=t)
+        torch.cuda.synchronize()
+        res.append((*part, tgt))
+    assert int(err.item()) == 0
+    for x, y in zip(*res):
+        assert torch.equal(x, y)
+    # fp32 sums of 72 products, ex2.approx and the fp32 logarithm of sums near 300: a few ulps of values near ten each
+    lse = (res[1][0].double() + res[1][1].double().log()).logsumexp(1)
+    assert float((lse - ref.logsumexp(1)).abs().max()) < 1e-4
