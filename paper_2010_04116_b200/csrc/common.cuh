@@ -381,6 +381,9 @@ inline bool dependent_launch_enabled() {
   return on;
 }
 
+// Kernels this host thread has launched (il_stats counts by it: several functions launch as many as the sizes ask for).
+inline thread_local long long kernels_launched = 0;
+
 // Launch with the grid's blocks grouped into clusters of `cluster` blocks (1: none).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dep_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster,
@@ -405,7 +408,9 @@ inline cudaError_t launch_dep_cluster(void (*kern)(KArgs...), dim3 grid, dim3 bl
   }
   cfg.attrs = at;
   cfg.numAttrs = n;
-  return cudaLaunchKernelEx(&cfg, kern, KArgs(std::forward<Args>(args))...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, KArgs(std::forward<Args>(args))...);
+  if (e == cudaSuccess) ++kernels_launched;
+  return e;
 }
 
 template <typename... KArgs, typename... Args>

@@ -305,7 +305,9 @@ il_status gemm(il_model* m, int k, const GemmArgs& g, cudaStream_t on = nullptr)
     }
     IL_CUDA(m, cudaEventRecord(rec.a, st));
   }
+  const long long l0 = kernels_launched;
   cudaError_t e = gemm_launch(g, m->err_word[k], m->sms[k], st);
+  m->launches += kernels_launched - l0;
   if (e != cudaSuccess)
     return fail(m, e == cudaErrorInvalidValue ? IL_ERR_INVALID_ARG : IL_ERR_CUDA, "gemm launch (M=%d N=%d K=%d epi=%d): %s",
                 g.M, g.N, g.K, g.epilogue, cudaGetErrorString(e));
@@ -316,7 +318,6 @@ il_status gemm(il_model* m, int k, const GemmArgs& g, cudaStream_t on = nullptr)
         if (j != k) IL_CUDA(m, cudaStreamWaitEvent(m->streams[j], rec.b, 0));
     m->prof_recs.push_back(rec);
   }
-  m->launches++;
   return IL_OK;
 }
 
@@ -332,11 +333,13 @@ GemmArgs gemm_args(int M, int N, int K, const void* A, int lda, int a_mn, const 
   return g;
 }
 
+// A function that launches kernels (one or several, counted as they are launched).
 #define IL_K(m, call)                                                                                   \
   do {                                                                                                  \
+    const long long l0__ = kernels_launched;                                                            \
     cudaError_t e__ = (call);                                                                           \
+    (m)->launches += kernels_launched - l0__;                                                           \
     if (e__ != cudaSuccess) return fail(m, IL_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e__));      \
-    (m)->launches++;                                                                                    \
   } while (0)
 
 // Weight-gradient GEMM dW[M,N] = dY^T X over K tokens.  The output has few tiles compared with the number of CTA
@@ -1275,7 +1278,6 @@ il_status layers_backward(il_model* m, int k, int s, size_t base, int count, con
     IL_TRY(br.join(1));                          // dbig (and, since the last block's mark came before, dqkv) is replaced
     IL_K(m, attention_bwd(A.qkv, A.attn_o, A.lse, c.dattn, c.dqkv, c.delta, dq_acc, s * m->B, m->B, m->T, m->H, m->dh,
                           m->err_word[k], st));
-    if (m->T > ATTN_BWD_SHORT_T) m->launches += 2;
     IL_TRY(br.fork());
     IL_K(m, colsum_bf16(c.dqkv, 3 * d, m->G[k] + o.bqkv, N, 3 * d, br.st));
     IL_TRY(wgrad(m, k, 3 * d, d, N, c.dqkv, 3 * d, A.ln1, d, m->G[k] + o.wqkv, acc, br.st));
@@ -1394,7 +1396,6 @@ il_status component_backward(il_model* m, int k, int s, bool acc, G&& gather) {
     if (k == 0) {
       IL_K(m, embed_bwd(m->tokens[k], m->sort_keys[0], m->cs[0].dx, m->G[k] + m->off_wte, m->G[k] + m->off_wpe, m->ntok, m->T, m->d,
                         m->V, acc ? 1 : 0, st));
-      m->launches++;
     }
     return IL_OK;
   });
