@@ -610,8 +610,11 @@ cudaError_t fwd_pair_launch(const bf16* qkv, bf16* o, float* lse, int B, int T, 
   if (!tma_encode_bf16(&tm, qkv, 4, dims, strides, box)) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(attn_fwd_pair_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const long long items = (long long)((T + 255) / 256) * B * H;
-  const int grid = (int)(items < 148 ? items : 148);
+  const int grid = (int)(items < sms ? items : sms);
   launch_dep(attn_fwd_pair_kernel<DH>, dim3(grid), dim3(FWD2_THREADS), C::SMEM, s, tm, o, lse, B, T, H, rsqrtf((float)DH), err);
   return cudaGetLastError();
 }
