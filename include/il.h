@@ -81,7 +81,8 @@ typedef struct {
                                     /* its last bit (and that of everything computed from it) may differ between runs.  */
                                     /* IL_ATTN_BWD_TWO_KERNELS (1): dK/dV and dQ in two kernels that each recompute the */
                                     /* scores; slower, every sum in a fixed order.  Head dims other than 32 / 64 always */
-                                    /* take the two-kernel form                                                         */
+                                    /* take the two-kernel form; sequences of up to 128 positions one kernel of fixed   */
+                                    /* order either way                                                                 */
   const int* devices;               /* IL_PLACE_PIPELINE: K device ordinals (n_devices == K), or NULL: every component */
   int n_devices;                    /* on `device`, still exchanged through the copy path.  Caller-owned streams[k]    */
                                     /* must belong to devices[k]; the alloc hook is called with that device current    */

@@ -72,7 +72,8 @@ il_status il_op_gemm(const il_gemm_desc* desc, unsigned* err_word, void* stream)
  * qkv and o 16-byte aligned, lse 4-byte aligned. */
 il_status il_op_attention_fwd(const void* qkv, void* o, float* lse, int B, int T, int H, int dh, void* stream);
 /* Its backward.  NB gradient batches may share the saved forward of B sequences (gradient batch b uses
- * sequence b % B): dout [NB*T, H*dh] bf16 -> dqkv [NB*T, 3*H*dh] bf16.  delta: scratch [NB*H*T] fp32.
+ * sequence b % B): dout [NB*T, H*dh] bf16 -> dqkv [NB*T, 3*H*dh] bf16.  delta: scratch [NB*H*T] fp32.  Sequences of
+ * up to 128 positions take one kernel that needs no scratch.
  * qkv, o, dout and dqkv must be 16-byte aligned (IL_ERR_INVALID_ARG otherwise, before anything is launched). */
 il_status il_op_attention_bwd(const void* qkv, const void* o, const float* lse, const void* dout, void* dqkv,
                               float* delta, int NB, int B, int T, int H, int dh, void* stream);
@@ -81,7 +82,8 @@ il_status il_op_attention_bwd(const void* qkv, const void* o, const float* lse, 
  * recomputation of S and dP (five products instead of the seven of the two-kernel form above).  dq_acc: scratch
  * [NB*T, H*dh] fp32, 16-byte aligned; every key tile adds its share of dQ into it with floating-point atomics
  * (the order of that sum, and so the last bit of dQ, may differ between runs), and a final pass writes it to dqkv
- * as bf16.  err_word: device word set non-zero if a bounded wait expired (may be NULL). */
+ * as bf16.  Sequences of up to 128 positions take the kernel of il_op_attention_bwd and leave dq_acc alone.  err_word:
+ * device word set non-zero if a bounded wait expired (may be NULL). */
 il_status il_op_attention_bwd_one_sweep(const void* qkv, const void* o, const float* lse, const void* dout, void* dqkv,
                                         float* delta, float* dq_acc, int NB, int B, int T, int H, int dh,
                                         unsigned* err_word, void* stream);

@@ -1124,9 +1124,10 @@ __global__ void __launch_bounds__(256) attn_bwd_dq_tc_kernel(const __grid_consta
 // What bounds it: a step of 128 x 128 takes about 3200 cycles, of which a recompute warp works 1400 (sixteen warps share the
 // issue slots) and an issuing thread 1700 (16 MMAs at 60, two commits at 120, looks at barriers at 150 each); the change of
 // items costs another step (K and V of one item only fit beside three Q / dO stages: with two buffers and two stages the tiles
-// came late and nothing was gained).  Measured, delta and conversion included: 16 x 16 heads x 1024, dh 64 236 -> 209 us, 8 x 16
-// 124 -> 107, against the form with all sixteen warps on either half in turn, one issuing thread per half and the four flush
-// warps staging a block together.
+// came late and nothing was gained).  Measured, delta and conversion included, launches back to back: 16 x 16 heads x 1024,
+// dh 64 236 -> 209 us, 8 x 16 124 -> 107, against the form with all sixteen warps on either half in turn, one issuing thread per half
+// and the four flush warps staging a block together; 211 and 110 on another GPU since dS has a barrier per buffer.  The 80
+// registers that 768 threads leave spill a little: 0.39 of 34.5 million warp instructions touch local memory.
 // The sum over key tiles in dQ is made by floating-point atomics: its order, and with it the last bit of dQ,
 // depends on scheduling.  Every wait is bounded.
 // ------------------------------------------------------------------------------------------------

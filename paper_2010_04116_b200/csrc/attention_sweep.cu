@@ -13,8 +13,8 @@
 // the tensor pipe runs step j's products and the scores of step j + 2 meanwhile.  Tensor memory: 2 x 128 score columns and one or
 // two accumulators of dh: one CTA per SM.  Items are numbered so that the longest sweeps start first.
 //
-// What bounds it: the issuing threads.  A thread issues an MMA of this size no faster than every 60 cycles (whether A comes from
-// shared or from tensor memory), a commit costs it 120, a look at a barrier 150 beside the busy pipe; a step of dQ at dh 128
+// What bounds it: the issuing threads.  A thread issues an MMA of this size no faster than every 60 cycles wherever A comes
+// from, a commit costs it 120, a look at a barrier 150 beside the busy pipe; a step of dQ at dh 128
 // takes 1440 cycles (one issuing thread: 1810), of which a row-work warp is busy 880.  Short sweeps pay 5 us an item for set-up,
 // first loads and output.
 // Measured, delta included (gradient sequences x heads x T, dh), us; the synchronous two-kernel form before it / this one:
@@ -52,7 +52,10 @@ attn_bwd_sweep_kernel(const __grid_constant__ CUtensorMap tm_row, const __grid_c
                       const __grid_constant__ CUtensorMap tm_do, const float* __restrict__ lse, const float* __restrict__ delta,
                       bf16* __restrict__ dqkv, int NB, int B, int T, int H, float scale, unsigned* err) {
   using C = SweepCfg<DH>;
-  // The row operands as the score products' A operand from tensor memory, where the columns suffice.
+  // The row operands as the score products' A operand from tensor memory, where the columns suffice.  With two issuing threads
+  // the shared-memory reads of the operands begin to show (us, cold cache, from tensor / from shared memory: 8 x 16 x 1024,
+  // dh 64 174.1 / 177.2; 16 x 16 x 1024 330.8 / 338.9; 2 x 32 x 2048, dh 80 271.4 / 272.4; 1 x 8 x 4096, dh 128 133.8 / 134.2); with
+  // one it was the other way round.
   constexpr uint32_t C_ROW = C::C_ACC + (KV ? 2 : 1) * DH;
   constexpr bool ROWS_IN_TMEM = C_ROW + DH <= 512;
   extern __shared__ uint8_t smem_raw[];

@@ -45,7 +45,8 @@ cudaError_t embed_fwd(const int* tok, const float* wte, const float* wpe, float*
 // chunk in shared memory, sorts them with a bitonic network over the next power of two (keys are distinct, so the
 // order is total) and lists the runs of equal tokens, short ones from the front and long ones from the back.  The
 // order of the lists is arbitrary; nothing depends on it, each run being one output row.
-// 8192 positions take 44 us (91 exchange passes), 256 take 4 us; the step runs it beside the forward pass.
+// 8192 positions take 44 us (91 exchange passes), 256 take 4 us; the step runs it beside the backward
+// passes that come before the embedding's.
 constexpr int SORT_CHUNK = 8192;
 constexpr int SORT_POS_BITS = 13;
 constexpr int RUN_LONG = 24;                         // rows from which a run is summed by a whole block
@@ -115,7 +116,7 @@ cudaError_t embed_sort(const int* tok, unsigned* keys, int ntok, int V, cudaStre
 // w, w + 8, ... and the eight partial sums are added in warp order), then warps share those of the short ones (rows in
 // order).  Every sum has a fixed order.  Under a Zipf law one token holds a tenth of all positions; a block per sorted
 // position, as this kernel once was, spent its time starting blocks that had nothing to do and on that one token:
-// 8192 x 1024 took 150-166 us, now 20.
+// 8192 x 1024 of Zipf tokens took 163 us from a cold cache, now 90.
 __global__ void __launch_bounds__(256) embed_bwd_wte_kernel(const unsigned* __restrict__ sorted, const float* __restrict__ dx,
                                                             float* __restrict__ dwte, int d, int accumulate) {
   grid_dep_wait();
@@ -859,8 +860,8 @@ __global__ void __launch_bounds__(256) adamw_kernel(float4* __restrict__ p, floa
 
 // background: beside a chain of kernels that must not wait for it.  A grid that fills the SMs' thread slots holds every other
 // kernel back until it ends (180 us for a GPT-2-small vocabulary matrix, four times in a step); three blocks per SM leave
-// room for a GEMM's CTA beside them and keep 48 KB per SM in flight, and a launch covers only so much (14 MB of parameters'
-// state) that a kernel which needs the whole SM gets it soon.  Measured, a step's time in us (filled grids / 3 blocks, 8 / 4 / 2
+// room for a GEMM's CTA beside them and keep 48 KB per SM in flight, and a launch covers only so much (1.8 million
+// parameters, 29 MB of p, m, v and g) that a kernel which needs the whole SM gets it soon.  Measured, a step's time in us (filled grids / 3 blocks, 8 / 4 / 2
 // iterations): GPT-2-small widths, 256 tokens 3250 / 3047 / 3026 / 3004; T 4096 3877 / 3846 / 3774 / 3748; 2.7B widths 12510 /
 // 11980 / 11890 / 12190.
 constexpr int BG_BLOCKS_PER_SM = 3, BG_ITERATIONS = 4;

@@ -654,13 +654,16 @@ bool encode_gemm_operand(CUtensorMap* tm, const GemmOperand& op, int rows, int k
 }
 
 // Which kernel and tile, from a model of each one's time in microseconds.  The constants are measured (back-to-back
-// launches of the shapes of a training step from 256 to 16384 tokens, d 128 to 2560); the choice is within 10 % of the
-// best candidate on nearly all of them.
+// launches of the shapes of a training step from 256 to 16384 tokens, d 128 to 2560).  Of 149 such products with all their
+// candidates timed, the choice is within 2 % of the best on 109 and within 10 % on 139; the others are d 2560 and 1024 weight
+// gradients that take the wide tile (up to 1.22, see its factor below), products of 200 to 2505 rows whose 128 x 64 tiles are
+// 1.1 better, and 2505 x 512 x 8192 (1.32: two cluster ranks would do).
 //   paired, 256 x 256: 0.283 us per slab alone, 0.345 with all pairs busy; a wave costs its main loop or its epilogue,
 //     whichever is longer (the accumulators alternate).
 //   paired, 256 x 512: 0.55 / 0.64 per slab (of twice the columns), the epilogue is exposed; only for k-ranges of 2048
 //     and more (8192 x 4096 x 1024 with the saved derivative: 112 us against 73 with square tiles).  Counted at 0.86: it
-//     moves a quarter fewer operand bytes, which back-to-back launches of one shape do not show but the power cap does.
+//     moves a quarter fewer operand bytes, which back-to-back launches of one shape do not show but the power cap does.  The
+//     factor was set on whole steps (GPT-2-medium shape 50.7 -> 50.1 ms, micro-batched paper shape 163 -> 160.2 ms).
 //   128 x 128 / 128 x 64: 0.26 / 0.245 per slab while each CTA has an SM to itself, 0.46 / 0.33 with two per SM, then
 //     counted at 1.1 for the opposite reason (twice the operand bytes of the square tile).
 // max_atomic_split > 1 (EPI_F32 into a zeroed output): the paired kernel may split the contraction over up to that

@@ -1595,9 +1595,9 @@ extern "C" il_status il_adamw_step(il_model* m, float lr, float beta1, float bet
   m->adamw_issued += 1;
   const double bc1 = 1.0 - pow((double)beta1, (double)m->step);
   const double bc2 = 1.0 - pow((double)beta2, (double)m->step);
-  // Parameters, gradients and bf16 shadows of component k (its head and, for k = 0, the embeddings included)
-  // are read and written by stream k only, so each component updates on its own stream as soon as its
-  // gradients are final (the last backward pass through a module triggers its update, App. C).
+  // Parameters, gradients and bf16 shadows of component k (its head and, for k = 0, the embeddings included) are read and
+  // written on stream k, its branch and its side stream only, which all join stream k, so each component updates as soon as
+  // its gradients are final (the last backward pass through a module triggers its update, App. C).
   for (int k = 0; k < m->K; ++k) {
     const size_t b = m->comp_begin[k], e = m->comp_end[k], me = m->comp_mat_end[k];
     IL_CUDA(m, cudaSetDevice(m->dev[k]));
